@@ -897,6 +897,8 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   const uint32_t n = (uint32_t)jobs.size();
   if (ws.pend.kind) return JIFFY_ERR_STATE;
   unsigned long long items = 0;
+  unsigned long long pixels = 0;
+  uint32_t chains = 0, max_T = 1;
   uint32_t max_W = 1;
   std::vector<jiffy_stream*> ss(n);
   for (uint32_t i = 0; i < n; i++) {
@@ -909,6 +911,9 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
     if (reinterpret_cast<uintptr_t>(j.in) & 3u) return JIFFY_ERR_INVALID_ARG;
     for (size_t q = 0; q < (size_t)j.T * s->A; q++)
       if (!j.planes_out[q]) return JIFFY_ERR_INVALID_ARG;
+    chains += s->A;
+    max_T = std::max(max_T, j.T);
+    pixels += (unsigned long long)j.T * s->A * s->H * s->W;
     if (j.async) {  // the offsets are on the device: the kernel checks them
       if (reinterpret_cast<uintptr_t>(j.frame_offsets) & 7u) return JIFFY_ERR_INVALID_ARG;
       items += (unsigned long long)j.T * s->A * s->H;
@@ -937,7 +942,8 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   if (items > 0x7fffffffull) return JIFFY_ERR_INVALID_ARG;
 
   Carver up;
-  const size_t u_seg = up.take(sizeof(jiffy::DecSeg) * n), u_ib = up.take(4ull * n), u_sb = up.take(4ull * n);
+  const size_t u_seg = up.take(sizeof(jiffy::DecSeg) * n), u_ib = up.take(4ull * n), u_sb = up.take(4ull * n),
+               u_cb = up.take(4ull * n);
   std::vector<size_t> u_ptrs(n);
   for (uint32_t i = 0; i < n; i++)
     u_ptrs[i] = up.take(8ull * ((size_t)(jobs[i].T + 2) * jobs[i].s->A + jobs[i].T + 1));
@@ -949,8 +955,7 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   const size_t o_up_slot[2] = {c.take(up.off), c.take(up.off)};
   const size_t o_up = o_up_slot[slot];
   const size_t o_zero = c.take(0);
-  const size_t o_done = c.take(4ull * items), o_tick = c.take(8);
-  const size_t o_res = c.take(rs.off);
+  const size_t o_done = c.take(4ull * items), o_tick = c.take(8), o_res = c.take(rs.off);
   const size_t zero_bytes = c.off - o_zero;
   std::vector<unsigned long long> mask_base(n);
   unsigned long long mask_words = 0;
@@ -959,14 +964,16 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
     mask_base[i] = mask_words;
     mask_words += (unsigned long long)jobs[i].T * s->A * s->H * ((s->W + 31) / 32);
   }
-  const size_t o_masks = c.take(4ull * mask_words);
+  const size_t o_masks = c.take(4ull * mask_words), o_chp = c.take(4ull * chains);
+  unsigned long long n_sec = 0;
+  for (uint32_t i = 0; i < n; i++) n_sec += (unsigned long long)jobs[i].T * jobs[i].s->A;
+  const size_t o_secs = c.take(sizeof(jiffy::DecSec) * n_sec);
   // Zstandard mask sections: their decoded (still XORed) mask bytes
   std::vector<unsigned long long> zm_base(n);
-  unsigned long long zm_total = 0, n_sec = 0;
+  unsigned long long zm_total = 0;
   uint32_t zmax_blk = 0;
   for (uint32_t i = 0; i < n; i++) {
     const jiffy_stream* s = jobs[i].s;
-    n_sec += (unsigned long long)jobs[i].T * s->A;
     if (!(s->opt.stages & jiffy::kStageZstdMask)) continue;
     zm_base[i] = zm_total;
     zm_total += align_up((size_t)s->H * ((s->W + 7) / 8), 16) * jobs[i].T * s->A;
@@ -983,10 +990,11 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   jiffy::DecSeg* segs = reinterpret_cast<jiffy::DecSeg*>(h + u_seg);
   uint32_t* ib = reinterpret_cast<uint32_t*>(h + u_ib);
   uint32_t* sbk = reinterpret_cast<uint32_t*>(h + u_sb);
+  uint32_t* cbk = reinterpret_cast<uint32_t*>(h + u_cb);
   std::vector<uint64_t> key{2, n, (uint64_t)(uintptr_t)d, (uint64_t)(uintptr_t)h};
   std::vector<uint32_t> sig{2, max_W, log2_ceil(items)};
   uint32_t staged = 0, withhold = 0;
-  uint32_t item_base = 0, sec_base = 0;
+  uint32_t item_base = 0, sec_base = 0, chain_base = 0;
   for (uint32_t i = 0; i < n; i++) {
     DecJob& j = jobs[i];
     jiffy_stream* s = j.s;
@@ -1017,7 +1025,9 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
     g.frame0 = s->frame;
     g.fhdr = frame_header_bytes(A);
     g.check_shdr = s->frame == 0;
+    g.clear_err = j.async ? 0u : 1u;  // (where nothing else clears it)
     g.item_base = item_base;
+    g.chain_base = chain_base;
     g.attrs = s->d_attrs;
     g.in = static_cast<const uint8_t*>(j.in);
     g.in_len = j.in_len;
@@ -1031,9 +1041,11 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
     segs[i] = g;
     ib[i] = item_base;
     sbk[i] = sec_base;
+    cbk[i] = chain_base;
     if (s->withhold < T * A * s->H) withhold = item_base + s->withhold + 1u;
     s->withhold = UINT32_MAX;  // one call
     item_base += T * A * s->H;
+    chain_base += A;
     sec_base += T * A;
     staged |= s->opt.stages ? 1u : 0u;
     key.push_back(((uint64_t)s->H << 32) | s->W);
@@ -1049,12 +1061,28 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   }
   key.push_back(async ? 1u : 0u);
 
+  // Small calls run the rows kernel alone: the kernels around it cost about
+  // 10 us a call (17 -> 28 us for 2 scans of 11 x 896, five attributes) and
+  // save a tenth of the rows' time, which is 10 us at some 16 million samples
+  // (100 scans of 128 x 2048, 131 million: 330 -> 290 us). They also take P
+  // runs apart, which pays for itself many times over in calls of many frames
+  // whose rows wait for one another (100 predicted scans of 64 x 489, 6
+  // million samples: 1.95 -> 0.12 ms), so long calls of a few thousand rows
+  // take them too.
+  const bool local = max_T == 1 || !(pixels >= (16ull << 20) || (max_T >= 32 && items >= 8192));
+
   jiffy::DecParams p{};
+  p.local = local ? 1u : 0u;
   p.n_seg = n;
   p.n_items = (uint32_t)items;
   p.max_W = max_W;
   p.seg = reinterpret_cast<const jiffy::DecSeg*>(d + o_up + u_seg);
   p.seg_item_base = reinterpret_cast<const uint32_t*>(d + o_up + u_ib);
+  p.secs = reinterpret_cast<jiffy::DecSec*>(d + o_secs);
+  p.n_chains = chains;
+  p.max_T = max_T;
+  p.seg_chain_base = reinterpret_cast<const uint32_t*>(d + o_up + u_cb);
+  p.chain_p = reinterpret_cast<uint32_t*>(d + o_chp);
   p.done = reinterpret_cast<uint32_t*>(d + o_done);
   p.masks = reinterpret_cast<uint32_t*>(d + o_masks);
   p.ticket = reinterpret_cast<uint32_t*>(d + o_tick);
@@ -1079,8 +1107,10 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   if (!up_same && async && record_ev(ws.uploaded, st) != cudaSuccess) return JIFFY_ERR_CUDA;
 
   auto enqueue = [&](cudaStream_t s, const jiffy::DecParams& pp, void* const* evs) -> int {
-    const cudaError_t ce = cudaMemsetAsync(d + o_zero, 0, zero_bytes, s);
-    if (ce != cudaSuccess) return (int)ce;
+    if (local) {
+      const cudaError_t ce = cudaMemsetAsync(d + o_zero, 0, zero_bytes, s);
+      if (ce != cudaSuccess) return (int)ce;
+    }
     const int rc = jiffy::launch_decode(pp, s, evs);
     if (rc != 0 || async) return rc;  // enqueue-only: errors stay on the device
     return (int)cudaMemcpyAsync(hres, d + o_res, rs.off, cudaMemcpyDeviceToHost, s);

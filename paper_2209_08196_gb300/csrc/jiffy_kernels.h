@@ -6,7 +6,8 @@
 // row r) and sections (scan t, attribute a) are numbered globally across the
 // segments of a call, segment after segment. Within a segment, sections are
 // ordered (t, a); the encoder's row items are ordered (a, t, r) (attribute-
-// major), and so are the decoder's.
+// major), and so are the decoder's. The attributes of the decoder's segments are
+// its chains: P frames chain the frames of an attribute.
 #pragma once
 
 #include <cstdint>
@@ -87,7 +88,9 @@ struct DecSeg {
   uint32_t frame0;
   uint32_t fhdr;
   uint32_t check_shdr;           // validate the stream header at in[0]
-  uint32_t item_base;
+  uint32_t clear_err;            // the error word belongs to this call: cleared first
+  uint32_t item_base;            // first global row item of the segment
+  uint32_t chain_base;           // first chain of the segment (it has A)
   const AttrDev* attrs;
   const uint8_t* in;
   unsigned long long in_len;
@@ -102,14 +105,35 @@ struct DecSeg {
   unsigned long long zm_base, zm_stride;  // its decoded mask bytes in DecParams::zdec
 };
 
+// A section of the call as found by the decoder's first kernel.
+struct alignas(16) DecSec {
+  unsigned long long sec;  // byte offset of the section (its row table)
+  uint32_t data_len;       // bytes of its row chunks
+  uint32_t zpart;          // bytes of the Zstandard mask part after the row table (0 without it)
+  uint32_t mode;           // 0 I, 1 P
+  uint32_t bad;            // 1: malformed frame or stream header
+  uint32_t link;           // how it is added to the frame before it in the call (kLink*), kLinkNext
+};
+
+// How the P frames of a chain are added to the frames before them: there are
+// none, their rows wait for the rows before, or k_dec_sums does it. kLinkNext:
+// the rows of the next frame wait for these.
+enum : uint32_t { kLinkNone = 0u, kLinkWait = 1u, kLinkSum = 2u, kLinkNext = 4u };
+
 struct DecParams {
   uint32_t n_seg;
   uint32_t n_items;
   uint32_t max_W;
   const DecSeg* seg;             // [n_seg]
   const uint32_t* seg_item_base; // [n_seg]
-  uint32_t* done;                // [n_items] row-done flags
-  uint32_t* masks;               // decoded zero masks, nw words per row item (read by the next frame's P rows)
+  uint32_t local;                // 1: a small call, the rows kernel alone (its ticket, error words and done flags zeroed)
+  DecSec* secs;                  // [n_sec] written by the call's first kernel
+  uint32_t n_chains;             // chains of all segments
+  const uint32_t* seg_chain_base;// [n_seg] (search key for chains)
+  uint32_t* chain_p;             // [n_chains] kLink* of the chain, by the call's first kernel
+  uint32_t max_T;                // most frames of a segment
+  uint32_t* done;                // [n_items] row-done flags (of the chains that wait)
+  uint32_t* masks;               // decoded zero masks, nw words per row item (frames coded P and those before them)
   uint32_t* ticket;
   uint32_t wpc;                  // warps per CTA (1, 2, 4, 8; 0 = by shared memory)
   uint32_t ctas_per_sm;          // resident CTAs per SM (0 = occupancy limit)
@@ -127,6 +151,7 @@ struct DecParams {
 // (requests clamped to what fits the device).
 struct RowsLaunch {
   uint32_t wpc, ctas_per_sm, items_per_ticket, grid;
+  uint32_t sms;  // of the device (decoder)
 };
 
 size_t enc_smem_bytes_host(uint32_t W);

@@ -747,6 +747,8 @@ __device__ bool read_stream(const ZDec& z, const uint8_t* s, uint32_t len, uint8
 
 __global__ void __launch_bounds__(32) k_zstd_dec(DecParams p) {
   __shared__ ZDec z;
+  chain_wait();
+  chain_start();
   const uint32_t gs = blockIdx.x, j = blockIdx.y, lane = threadIdx.x;
   const DecSeg& sg = p.seg[sec_segment(p.seg_sec_base, p.n_seg, gs)];
   if (!(sg.stages & kStageZstdMask) || j >= sg.zm_nblk) return;
@@ -910,8 +912,7 @@ int launch_zstd_encode(const EncParams& p, void* stream) {
 int launch_zstd_decode(const DecParams& p, void* stream) {
   if (!p.zdec || !p.zmax_blk) return 0;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  k_zstd_dec<<<dim3(p.n_sec, p.zmax_blk), 32, 0, st>>>(p);
-  return (int)cudaGetLastError();
+  return (int)launch_chained(k_zstd_dec, dim3(p.n_sec, p.zmax_blk), 32u, 0, st, p);
 }
 
 }  // namespace jiffy
