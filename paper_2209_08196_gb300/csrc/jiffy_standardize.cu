@@ -63,6 +63,7 @@ struct StdParams {
   uint32_t az0;          // binary angle (2^32 per turn)
   int top, bottom;       // elevation limits (H > 1)
   const int* mid;        // [H - 1] midpoints between beams, decreasing
+  float el0, row_scale;  // row of elevation el, were the beams evenly spaced: (el0 - el) row_scale
   int atan_t[kStdIter];
   const float* xyz;
   unsigned long long* keys;  // [T][H * W]
@@ -71,8 +72,7 @@ struct StdParams {
   unsigned long long off[kStdMaxScans + 1];  // scan t's points: [off[t], off[t + 1])
 };
 
-__device__ __forceinline__ bool coord(float v, float k, long long& out) {
-  const float p = __fmul_rn(v, k);
+__device__ __forceinline__ bool coord(float p, long long& out) {
   if (!(fabsf(p) < 2147483648.0f)) return false;  // also NaN
   out = (long long)rintf(p);                     // round half to even
   return true;
@@ -149,63 +149,158 @@ __device__ __forceinline__ uint32_t quantize_attr(float v, float scale, uint32_t
   return r >= (float)mx ? mx : (uint32_t)r;
 }
 
+// Square root to 2^-23 relative.
+__device__ __forceinline__ float root(float v) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+
+// The exact pixel of a point in range (row * W + column; ~0 outside the
+// vertical field of view), by CORDIC: the definition, taken for the points
+// that quick_pixel leaves open.
+__device__ __noinline__ uint32_t exact_pixel(const StdParams& p, long long X, long long Y, long long Z) {
+  const int* t = p.atan_t;
+  uint32_t row = 0;
+  if (p.H > 1) {
+    const int el = elevation(X, Y, Z, t);
+    if (el > p.top || el < p.bottom) return ~0u;
+    uint32_t lo = 0, hi = p.H - 1;  // row = number of midpoints above el
+    while (lo < hi) {
+      const uint32_t m = (lo + hi) >> 1;
+      if (__ldg(p.mid + m) > el) lo = m + 1;
+      else hi = m;
+    }
+    row = lo;
+  }
+  const uint32_t a = azimuth(X, Y, t) - p.az0;  // modulo 2^32
+  return row * p.W + (uint32_t)(((unsigned long long)a * p.W) >> 32);
+}
+
+// The same pixel from float32 angles, where they decide it. A CORDIC angle is
+// within 1.5e-7 rad of the true one (30 truncated steps on 28-bit vectors and
+// more, 30 rounded table entries), a float32 one within 1.2e-6 rad (atan2f: 3
+// ulp, 7.2e-7 at half a turn; inputs and scaling 4e-7): together less than
+// 1000 units of 2^-32 turn. So where the pixel is the same over kMargin units
+// either side of the float angle, the CORDIC angle falls into it too. About 1
+// point in 300 of a 128 x 2048 image is closer to an edge than that (returns
+// false) and goes to exact_pixel. With two CORDICs for every point (935
+// instructions) the kernel was bound by issue: 273 us for 40 scans of
+// 128 x 2048, 74 us this way.
+constexpr int kMargin = 2048;
+constexpr float kUnits = 683565275.576f;  // 2^32 / (2 pi)
+
+__device__ __forceinline__ bool quick_pixel(const StdParams& p, float x, float y, float z, uint32_t& px) {
+  uint32_t row = 0;
+  if (p.H > 1) {
+    const int el = __float2int_rn(atan2f(z, root(x * x + y * y)) * kUnits);  // |el| <= 2^30
+    if (el - kMargin > p.top || el + kMargin < p.bottom) {
+      px = ~0u;
+      return true;
+    }
+    if (el + kMargin > p.top || el - kMargin < p.bottom) return false;
+    auto above = [&](uint32_t m) { return __ldg(p.mid + m) > el; };
+    // evenly spaced beams: the row directly, else by search
+    uint32_t lo = (uint32_t)min(max(__float2int_rn((p.el0 - (float)el) * p.row_scale), 0), (int)p.H - 1);
+    if ((lo > 0 && !above(lo - 1u)) || (lo < p.H - 1u && above(lo))) {
+      uint32_t hi = p.H - 1;
+      lo = 0;
+      while (lo < hi) {
+        const uint32_t m = (lo + hi) >> 1;
+        if (above(m)) lo = m + 1;
+        else hi = m;
+      }
+    }
+    if ((lo > 0 && __ldg(p.mid + lo - 1u) <= el + kMargin) || (lo < p.H - 1u && __ldg(p.mid + lo) > el - kMargin))
+      return false;
+    row = lo;
+  }
+  const uint32_t a = (uint32_t)__float2int_rn(atan2f(y, x) * kUnits) - p.az0;  // modulo 2^32
+  const uint32_t a0 = a - kMargin, a1 = a + kMargin, col = __umulhi(a0, p.W);
+  if (a0 > a1 || __umulhi(a1, p.W) != col) return false;
+  px = row * p.W + col;
+  return true;
+}
+
 __global__ void __launch_bounds__(256) k_std_points(const __grid_constant__ StdParams p) {
-  __shared__ int t[kStdIter];
-  for (int i = threadIdx.x; i < kStdIter; i += blockDim.x) t[i] = p.atan_t[i];
-  __syncthreads();
   const uint32_t scan = blockIdx.y;
   const unsigned long long p0 = p.off[scan], n = p.off[scan + 1] - p0;
   unsigned long long* keys = p.keys + (size_t)scan * p.H * p.W;
   for (unsigned long long ii = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; ii < n;
        ii += (unsigned long long)gridDim.x * blockDim.x) {
     const uint32_t i = (uint32_t)ii;  // index within the scan (< 2^32)
-    long long X, Y, Z;
     const float* q = p.xyz + 3ull * (p0 + ii);
-    if (!coord(__ldg(q), p.k, X) || !coord(__ldg(q + 1), p.k, Y) || !coord(__ldg(q + 2), p.k, Z)) continue;
-    if (p.clockwise) Y = -Y;
-    const unsigned long long n = (unsigned long long)(X * X) + (unsigned long long)(Y * Y) +
-                                 (unsigned long long)(Z * Z);  // < 3 2^62
-    const unsigned long long r = isqrt64(n);
-    const unsigned long long R = r + ((n - r * r) > r ? 1ull : 0ull);
-    if (R < 1 || R < p.rmin || R > p.rmax) continue;
-    uint32_t row = 0;
-    if (p.H > 1) {
-      const int el = elevation(X, Y, Z, t);
-      if (el > p.top || el < p.bottom) continue;
-      uint32_t lo = 0, hi = p.H - 1;  // row = number of midpoints above el
-      while (lo < hi) {
-        const uint32_t m = (lo + hi) >> 1;
-        if (__ldg(p.mid + m) > el) lo = m + 1;
-        else hi = m;
-      }
-      row = lo;
+    const float fx = __fmul_rn(__ldg(q), p.k), fy = __fmul_rn(__ldg(q + 1), p.k), fz = __fmul_rn(__ldg(q + 2), p.k);
+    unsigned long long R;
+    uint32_t px;
+    if (fmaxf(fmaxf(fabsf(fx), fabsf(fy)), fabsf(fz)) < 1048576.0f && fx == fx && fy == fy && fz == fz) {
+      // |X|, |Y|, |Z| <= 2^20, exact in float32: the range from a float32
+      // root off by less than 1.5 and one correction against the sum of
+      // squares modulo 2^32
+      const int X = __float2int_rn(fx), Z = __float2int_rn(fz), Y = p.clockwise ? -__float2int_rn(fy) : __float2int_rn(fy);
+      const float x = (float)X, y = (float)Y, z = (float)Z;
+      int r = __float2int_rn(root(x * x + y * y + z * z));
+      auto sq = [](int v) { return (uint32_t)v * (uint32_t)v; };
+      const int e = (int)(sq(X) + sq(Y) + sq(Z) - sq(r));
+      if (e > r) r++;
+      else if (e <= -r) r--;
+      R = (unsigned long long)(uint32_t)r;
+      if (r < 1 || (uint32_t)r < p.rmin || (uint32_t)r > p.rmax) continue;
+      if (!quick_pixel(p, x, y, z, px)) px = exact_pixel(p, X, Y, Z);
+    } else {
+      long long X, Y, Z;
+      if (!coord(fx, X) || !coord(fy, Y) || !coord(fz, Z)) continue;
+      if (p.clockwise) Y = -Y;
+      const unsigned long long m = (unsigned long long)(X * X) + (unsigned long long)(Y * Y) +
+                                   (unsigned long long)(Z * Z);  // < 3 2^62
+      const unsigned long long r = isqrt64(m);
+      R = r + ((m - r * r) > r ? 1ull : 0ull);
+      if (R < 1 || R < p.rmin || R > p.rmax) continue;
+      px = exact_pixel(p, X, Y, Z);
     }
-    const uint32_t a = azimuth(X, Y, t) - p.az0;  // modulo 2^32
-    const uint32_t col = (uint32_t)(((unsigned long long)a * p.W) >> 32);
-    atomicMin(keys + (size_t)row * p.W + col, (R << 32) | i);
+    if (px != ~0u) atomicMin(keys + px, (R << 32) | i);
   }
 }
 
+// One pixel of every scan: a warp takes 128 pixels of a scan at a time, each
+// lane four of them 32 apart, so that four keys and then four values per
+// attribute are in flight and every access of a warp is to neighbouring
+// words (40 scans of 128 x 2048 with three attributes: 68 us; one pixel per lane
+// took 92, four neighbouring ones as vectors 177). Bound by memory: the keys
+// in and out, the winners' attributes, the images.
 __global__ void __launch_bounds__(256) k_std_pixels(const __grid_constant__ StdParams p) {
-  const uint32_t HW = p.H * p.W;  // <= 2^26
-  const size_t total = (size_t)HW * p.T;
-  const uint32_t G = gridDim.x * blockDim.x, g0 = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t dt = G / HW, dr = G % HW;  // the stride as (scans, pixels)
-  uint32_t t = g0 / HW, r = g0 % HW;        // this thread's scan and pixel
-  for (size_t px = g0; px < total; px += G) {
-    const unsigned long long key = p.keys[px];
-    const bool hit = key != ~0ull;
-    if (hit) p.keys[px] = ~0ull;  // ready for the next call
-    const unsigned long long idx = p.off[t] + (uint32_t)key;  // the point, across the call
-    store_sample(p.range_out, p.range_bytes, px, hit ? (uint32_t)(key >> 32) : 0u);
+  constexpr uint32_t N = 4;
+  const uint32_t HW = p.H * p.W, tiles = (HW + 127u) / 128u;  // HW <= 2^26
+  const uint32_t lane = threadIdx.x & 31u, G = gridDim.x * 8u, g0 = blockIdx.x * 8u + (threadIdx.x >> 5);
+  const uint32_t dt = G / tiles, dr = G % tiles;  // the stride as (scans, tiles)
+  uint32_t t = g0 / tiles, r = g0 % tiles;        // this warp's scan and tile
+  while (t < p.T) {
+    const uint32_t px = 128u * r + lane;
+    const size_t at0 = (size_t)t * HW + px;
+    unsigned long long key[N];
+#pragma unroll
+    for (uint32_t i = 0; i < N; i++) key[i] = px + 32u * i < HW ? p.keys[at0 + 32u * i] : ~0ull;
+    const unsigned long long first = p.off[t];
+#pragma unroll
+    for (uint32_t i = 0; i < N; i++) {
+      if (px + 32u * i >= HW) continue;
+      const bool hit = key[i] != ~0ull;
+      if (hit) p.keys[at0 + 32u * i] = ~0ull;  // ready for the next call
+      store_sample(p.range_out, p.range_bytes, at0 + 32u * i, hit ? (uint32_t)(key[i] >> 32) : 0u);
+    }
     for (uint32_t a = 0; a < p.n_attr; a++) {
       const StdAttr& at = p.attr[a];
-      store_sample(at.out, at.bytes, px, hit ? quantize_attr(__ldg(at.v + idx), at.scale, at.bytes) : 0u);
+      float f[N];  // the winning points' values
+#pragma unroll
+      for (uint32_t i = 0; i < N; i++) f[i] = key[i] != ~0ull ? __ldg(at.v + first + (uint32_t)key[i]) : 0.0f;
+#pragma unroll
+      for (uint32_t i = 0; i < N; i++)
+        if (px + 32u * i < HW) store_sample(at.out, at.bytes, at0 + 32u * i, quantize_attr(f[i], at.scale, at.bytes));  // (0 gives 0)
     }
     t += dt;
     r += dr;
-    if (r >= HW) {
-      r -= HW;
+    if (r >= tiles) {
+      r -= tiles;
       t++;
     }
   }
@@ -269,6 +364,8 @@ jiffy_status jiffy_standardizer_create(jiffy_standardizer** out, const jiffy_sen
     if (H > 1) {
       p.top = (int)std::min<long long>(alt[0] + (alt[0] - alt[1]) / 2, 0x7fffffffll);
       p.bottom = (int)std::max<long long>(alt[H - 1] - (alt[H - 2] - alt[H - 1]) / 2, -0x7fffffffll - 1);
+      p.el0 = (float)alt[0];
+      p.row_scale = (float)((double)(H - 1) / (double)(alt[0] - alt[H - 1]));
     }
     for (int i = 0; i < kStdIter; i++)
       p.atan_t[i] = (int)std::llround(std::atan(std::ldexp(1.0, -i)) / (2.0 * kPi) * 4294967296.0);
@@ -357,7 +454,8 @@ jiffy_status jiffy_standardize_seq(jiffy_standardizer* s, uint32_t n_scans, cons
           1ull, std::min<unsigned long long>(need, (target + n_scans - 1) / n_scans));
       k_std_points<<<dim3(bx, n_scans), 256, 0, st>>>(p);
     }
-    k_std_pixels<<<(uint32_t)std::min<size_t>(target, (HW * n_scans + 255) / 256), 256, 0, st>>>(p);
+    const size_t tiles = (HW + 127) / 128 * n_scans;
+    k_std_pixels<<<(uint32_t)std::min<size_t>(target, (tiles + 7) / 8), 256, 0, st>>>(p);
     if (cudaGetLastError() != cudaSuccess) rc = JIFFY_ERR_CUDA;
   }
   cudaSetDevice(prev);

@@ -184,3 +184,46 @@ def test_invalid_sensors_are_rejected():
         J.jiffy_standardizer_create(4, 16, beams(4), units_per_m=0.0)
     with pytest.raises(J.JiffyError):  # beyond +-90 degrees
         J.jiffy_standardizer_create(3, 16, [1.7, 0.0, -0.1])
+
+
+@pytest.mark.parametrize("H,W,kw", [
+    (128, 2048, {}), (5, 331, {"clockwise": True, "azimuth0": 0.3}), (1, 16384, {}), (64, 16384, {"azimuth0": math.pi}),
+    (16, 3, {"range_bytes": 2}), (40, 1024, {"units_per_m": 250.0}),
+])
+def test_points_close_to_pixel_edges(H, W, kw):
+    # within some 1e-7 to 1e-5 rad of the azimuth and elevation edges of the
+    # pixels, where float32 angles cannot decide, and of the vertical field of
+    # view; evenly and unevenly spaced beams; coordinates past the float32
+    # path's 2^20 units as well
+    rng = np.random.default_rng(H * W)
+    n = 20_000
+    for alt in (beams(H), np.sort(np.radians(rng.uniform(-40.0, 40.0, H)))[::-1]):
+        mids = np.concatenate([[alt[0] + 0.01], (alt[1:] + alt[:-1]) / 2, [alt[-1] - 0.01]]) if H > 1 else np.array([0.0])
+        if H > 1:
+            mids[0], mids[-1] = alt[0] + (alt[0] - alt[1]) / 2, alt[-1] - (alt[-2] - alt[-1]) / 2
+        near = 10.0 ** rng.uniform(-9, -5, size=(2, n)) * rng.choice([-1, 1], size=(2, n))
+        az = rng.integers(0, W, n) * (2 * math.pi / W) + kw.get("azimuth0", 0.0) + near[0]
+        el = np.clip(mids[rng.integers(0, len(mids), n)] + near[1], -1.5, 1.5)
+        d = rng.choice([0.05, 3.0, 60.0, 900.0, 1500.0, 9000.0], n) * rng.uniform(0.7, 1.0, n)
+        if kw.get("clockwise"):
+            az = -az
+        xyz = np.stack([d * np.cos(el) * np.cos(az), d * np.cos(el) * np.sin(az), d * np.sin(el)], 1).astype(np.float32)
+        xyz[:40] *= np.array([[0.0, 1.0, 0.0]], np.float32)  # on the axes, signed zeros among them
+        xyz[40:80] *= np.array([[-1.0, 0.0, 0.0]], np.float32)
+        xyz[80:120] *= np.array([[0.0, -0.0, 1.0]], np.float32)
+        check(xyz, H, W, alt, attrs=[(rng.uniform(0, 300, n), 2, 1.0), (rng.uniform(0, 300, n), 1, 1.0)], **kw)
+
+
+def test_range_rounding_around_half_units():
+    # the nearest integer to the root around every k + 1/2, up to the float32
+    # path's limit and past it
+    r = np.concatenate([np.arange(1, 4000), np.arange(1 << 20, (1 << 20) + 300), np.arange(1 << 21, (1 << 21) + 300),
+                        np.array([1_815_000, 1_816_000])])
+    H, W = 1, 4096
+    for seed in range(4):
+        rng = np.random.default_rng(seed)
+        az = rng.uniform(0, 2 * math.pi, len(r))
+        el = rng.uniform(-0.4, 0.4, len(r))
+        d = r + 0.5 + rng.uniform(-1e-3, 1e-3, len(r))
+        xyz = np.stack([d * np.cos(el) * np.cos(az), d * np.cos(el) * np.sin(az), d * np.sin(el)], 1).astype(np.float32)
+        check(xyz, H, W, np.zeros(1), units_per_m=1.0)
