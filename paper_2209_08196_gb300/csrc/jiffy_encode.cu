@@ -122,13 +122,19 @@ __device__ __forceinline__ uint32_t zigzag_small(uint32_t d) {
   return min(t, 1u - t);
 }
 
+// (precisions without a 32-bit multiplier, out of line: 64-bit products)
+__device__ __noinline__ uint32_t quant_wide(uint32_t v, const AttrDev& at) { return quant<2>(v, at); }
+__device__ __forceinline__ void quant8_wide(uint32_t (&v)[8], const AttrDev& at) {
+#pragma unroll
+  for (int i = 0; i < 8; i++) v[i] = quant_wide(v[i], at);
+}
+
 __device__ __forceinline__ void quant8(uint32_t (&v)[8], const AttrDev& at) {
   if (at.qkind == 1) {
 #pragma unroll
     for (int i = 0; i < 8; i++) v[i] = quant<1>(v[i], at);
   } else if (at.qkind == 2) {
-#pragma unroll
-    for (int i = 0; i < 8; i++) v[i] = quant<2>(v[i], at);
+    quant8_wide(v, at);
   }
 }
 
@@ -138,7 +144,7 @@ __device__ __forceinline__ void quant8(uint32_t (&v)[8], const AttrDev& at) {
 // q, P with prv: q - q', Sec. III-D) go to zb in row-major order (padded
 // layout), the coded mask bytes (M, or M xor M_prev for P, Sec. III-C/D) to
 // mb. qhi receives the largest quantized sample of the row (current and
-// previous scan) for 4-byte samples (0 otherwise). One copy of the code
+// previous scan) for 4-byte samples (0 otherwise). The trial uses it too. One copy of the code
 // serves every sample width, quantizer and mode (warp-uniform branches
 // around small blocks): the kernel is bound by instruction fetch, so its
 // footprint matters more than a few uniform branches per step.
@@ -149,6 +155,7 @@ __device__ __forceinline__ uint32_t pass_a(const uint8_t* cur, const uint8_t* pr
   const bool vc = vec_ok(cur, s), vp = prv && vec_ok(prv, s);
   const uint32_t Wm = (W + 31u) & ~31u;
   uint32_t n = 0, qm = 0;
+#pragma unroll 1
   for (uint32_t base = 0; base < W; base += kStepPx) {
     const uint32_t x0 = base + 8u * lane;
     const uint32_t nv = x0 < W ? min(8u, W - x0) : 0u;
@@ -199,6 +206,7 @@ __device__ __forceinline__ uint32_t pass_a(const uint8_t* cur, const uint8_t* pr
 __device__ __noinline__ void state_row(const uint8_t* cur, uint8_t* st_row, const AttrDev at, uint32_t W) {
   const uint32_t lane = lane_id(), s = at.s;
   const bool vc = vec_ok(cur, s), vs = vec_ok(st_row, s);
+#pragma unroll 1
   for (uint32_t base = 0; base < W; base += kStepPx) {
     const uint32_t x0 = base + 8u * lane;
     const uint32_t nv = x0 < W ? min(8u, W - x0) : 0u;
@@ -210,42 +218,6 @@ __device__ __noinline__ void state_row(const uint8_t* cur, uint8_t* st_row, cons
     for (int i = 0; i < 8; i++) v[i] *= at.P;
     store8(st_row, s, x0, nv, vs, v);
   }
-}
-
-// Pass A of the trial: the residuals of the row's kept samples both ways (I
-// to zi, P to zp).
-template <int QU>
-__device__ __forceinline__ uint32_t pass_a_trial(const uint8_t* cur, const uint8_t* prv, const AttrDev at, uint32_t W,
-                                              uint32_t kz, bool pmode, uint32_t* zb) {
-  const uint32_t lane = lane_id(), S = at.s;
-  const bool vc = vec_ok(cur, S), vp = vec_ok(prv, S);
-  uint32_t n = 0;
-  for (uint32_t base = 0; base < W; base += kStepPx) {
-    const uint32_t x0 = base + 8u * lane;
-    const uint32_t nv = x0 < W ? min(8u, W - x0) : 0u;
-    uint32_t v[8], pv[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    load8<false>(cur, S, x0, nv, vc, v);
-    if (pmode) load8<false>(prv, S, x0, nv, vp, pv);
-    uint32_t zm = 0;
-#pragma unroll
-    for (int i = 0; i < 8; i++) {
-      v[i] = quant<QU>(v[i], at);
-      if (pmode) pv[i] = v[i] - quant<QU>(pv[i], at);
-      zm |= (v[i] == 0u ? 1u : 0u) << i;
-    }
-    const uint32_t nz = ~(zm & kz) & ((1u << nv) - 1u);
-    uint32_t tot;
-    uint32_t kk = n + warp_excl_scan(__popc(nz), tot);
-#pragma unroll
-    for (int i = 0; i < 8; i++) {
-      if ((nz >> i) & 1u) {
-        zb[zaddr(kk)] = pmode ? pv[i] : v[i];
-        kk++;
-      }
-    }
-    n += tot;
-  }
-  return n;
 }
 
 // The residuals (I and, with prv, P) of the last nonzero sample (with all,
@@ -290,56 +262,82 @@ __device__ __noinline__ bool row_last(const uint8_t* cur, const uint8_t* prv, co
 // they count as zero-width values.
 __device__ __forceinline__ void fill_tail(uint32_t* zb, uint32_t n, uint32_t last) {
   const uint32_t end = (n + kStepVal - 1) / kStepVal * kStepVal;
+#pragma unroll 1
   for (uint32_t k = n + lane_id(); k < end; k += 32u) zb[zaddr(k)] = last;
   __syncwarp();
 }
 
 // ---------------------------------------------------------------------------
-// Block width (Sec. II, PFOR): b in [0, wmax] minimising the block's body
-// bytes, ties to the smallest b. Warp-wide: lane l holds the 32 consecutive
-// values z of its segment, the 4 lanes 4g'..4g'+3 (j = l & 3) hold one block
-// of m values (the values past m are 0). For each value, its unary width
-// code has bit b set iff the value needs more than b bits, so the column
-// sums of a block's unary codes are e_b = #values wider than b, for all b at
-// once: carry-save adders give each lane its 6 bit planes (counts <= 32),
-// two bit-sliced additions across the block's 4 lanes give 8 planes (counts
-// <= 128). Each lane then prices the candidates b = j, j+4, ... Returns
-// f << 14 | b << 8 | e (f = body bytes), the same in the block's 4 lanes
-// (all ones for m = 0); wmax = the bits of the block's widest value.
+// Delta (Sec. III-C) and ZigZag (Eq. 1) of a lane's 32 consecutive residuals,
+// in place in shared memory (zs; pred = the residual before the first), and
+// the column counts of the values' unary width codes: a value's code has bit
+// b set iff the value needs more than b bits, so that the counts of a block
+// are e_b = #values wider than b for all b at once; carry-save adders keep
+// them as 6 bit planes (counts <= 32). DELTA off: zs holds the values to pack
+// already. Eight values per turn of a rolled loop: all 32 in registers, with
+// the packing below unrolled as well, made the kernel 4900 instructions long,
+// executed about once per row, and instruction fetch its first stall.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t block_width(const uint32_t (&z)[32], uint32_t j, uint32_t m, uint32_t& wmax) {
-  // per-lane column counts of the unary width codes: 6 bit planes
-  uint32_t p1, p2, p4, p8, p16, p32;
-  {
-    uint32_t ones = 0, twos = 0, fours = 0, eights = 0, sixteens[2];
+template <bool DELTA>
+__device__ __forceinline__ void seg_planes(uint32_t* zs, uint32_t pred, uint32_t (&P)[6]) {
+  uint4* sp = reinterpret_cast<uint4*>(zs);
+  uint32_t ones = 0, twos = 0, fours = 0, eights = 0, sixteens = 0, thirtytwos = 0;
+#pragma unroll 1
+  for (uint32_t g = 0; g < 4; g++) {
+    const uint4 x = sp[2 * g], y = sp[2 * g + 1];
+    uint32_t z[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+    if (DELTA) {
+      const uint32_t last = z[7];
 #pragma unroll
-    for (int h = 0; h < 2; h++) {
-      uint32_t ta, tb, fa, fb, ea, eb;
-      const int o = 16 * h;
-      csa(ta, ones, ones, width_unary(z[o + 0]), width_unary(z[o + 1]));
-      csa(tb, ones, ones, width_unary(z[o + 2]), width_unary(z[o + 3]));
-      csa(fa, twos, twos, ta, tb);
-      csa(ta, ones, ones, width_unary(z[o + 4]), width_unary(z[o + 5]));
-      csa(tb, ones, ones, width_unary(z[o + 6]), width_unary(z[o + 7]));
-      csa(fb, twos, twos, ta, tb);
-      csa(ea, fours, fours, fa, fb);
-      csa(ta, ones, ones, width_unary(z[o + 8]), width_unary(z[o + 9]));
-      csa(tb, ones, ones, width_unary(z[o + 10]), width_unary(z[o + 11]));
-      csa(fa, twos, twos, ta, tb);
-      csa(ta, ones, ones, width_unary(z[o + 12]), width_unary(z[o + 13]));
-      csa(tb, ones, ones, width_unary(z[o + 14]), width_unary(z[o + 15]));
-      csa(fb, twos, twos, ta, tb);
-      csa(eb, fours, fours, fa, fb);
-      csa(sixteens[h], eights, eights, ea, eb);
+      for (int i = 7; i >= 0; i--) z[i] = zigzag_small(z[i] - (i ? z[i - 1] : pred));
+      pred = last;
+      sp[2 * g] = make_uint4(z[0], z[1], z[2], z[3]);
+      sp[2 * g + 1] = make_uint4(z[4], z[5], z[6], z[7]);
     }
-    p1 = ones; p2 = twos; p4 = fours; p8 = eights;
-    p16 = sixteens[0] ^ sixteens[1];
-    p32 = sixteens[0] & sixteens[1];
+    uint32_t ta, tb, fa, fb, e;
+    csa(ta, ones, ones, width_unary(z[0]), width_unary(z[1]));
+    csa(tb, ones, ones, width_unary(z[2]), width_unary(z[3]));
+    csa(fa, twos, twos, ta, tb);
+    csa(ta, ones, ones, width_unary(z[4]), width_unary(z[5]));
+    csa(tb, ones, ones, width_unary(z[6]), width_unary(z[7]));
+    csa(fb, twos, twos, ta, tb);
+    csa(e, fours, fours, fa, fb);
+    const uint32_t c = eights & e, c2 = sixteens & c;
+    eights ^= e;
+    sixteens ^= c;
+    thirtytwos ^= c2;
   }
+  P[0] = ones; P[1] = twos; P[2] = fours; P[3] = eights; P[4] = sixteens; P[5] = thirtytwos;
+}
+
+// The same for any deltas and for ablated codecs (Sec. IV-H): one value at a
+// time (rare), then the planes.
+__device__ __noinline__ void seg_delta_any(uint32_t* zs, uint32_t pred, uint32_t st) {
+  uint32_t prev = pred;
+#pragma unroll 1
+  for (uint32_t i = 0; i < 32; i++) {
+    const uint32_t e = zs[i];
+    const uint32_t d = (st & kStageNoDelta) ? e : e - prev;
+    zs[i] = (st & kStageNoZigzag) ? d : zigzag(d);
+    prev = e;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Block width (Sec. II, PFOR): b in [0, wmax] minimising the block's body
+// bytes, ties to the smallest b. Warp-wide: lane l holds the column counts of
+// the 32 values of its segment (seg_planes), the 4 lanes 4g'..4g'+3 (j = l &
+// 3) one block of m values (the values past m are 0): two bit-sliced additions
+// across the block's 4 lanes give 8 planes (counts <= 128). Each lane then
+// prices the candidates b = j, j+4, ... Returns f << 14 | b << 8 | e (f = body
+// bytes), the same in the block's 4 lanes (all ones for m = 0); wmax = the
+// bits of the block's widest value.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t block_width(const uint32_t (&A)[6], uint32_t j, uint32_t m, uint32_t& wmax) {
   // bit-sliced sums across the block's 4 lanes: 8 planes E[0..7]
   uint32_t E[8];
   {
-    uint32_t A[6] = {p1, p2, p4, p8, p16, p32}, B[7];
+    uint32_t B[7];
 #pragma unroll
     for (int k = 0; k < 6; k++) B[k] = __shfl_xor_sync(kFull, A[k], 1);
     uint32_t C[7], c = 0;
@@ -393,55 +391,39 @@ __device__ __forceinline__ uint32_t block_width(const uint32_t (&z)[32], uint32_
   return key;
 }
 
-// Delta (Sec. III-C) and ZigZag (Eq. 1) of a lane's 32 consecutive residuals
-// in place; pred = the residual before the first. FAST: every delta is below
-// 2^30 in magnitude (zigzag_small). st: stage switches (delta and ZigZag may
-// be off, Sec. IV-H).
-template <bool STAGED, bool FAST>
-__device__ __forceinline__ void delta_zigzag(uint32_t (&z)[32], uint32_t pred, uint32_t st) {
-  if (!STAGED || !(st & (kStageNoDelta | kStageNoZigzag))) {
-#pragma unroll
-    for (int i = 31; i >= 0; i--) {
-      const uint32_t d = z[i] - (i ? z[i - 1] : pred);
-      z[i] = FAST ? zigzag_small(d) : zigzag(d);
-    }
-  } else {  // ablated codecs (Sec. IV-H); values past n are 0 without the delta
-#pragma unroll
-    for (int i = 31; i >= 0; i--) {
-      const uint32_t d = (st & kStageNoDelta) ? z[i] : z[i] - (i ? z[i - 1] : pred);
-      z[i] = (st & kStageNoZigzag) ? d : zigzag(d);
-    }
-  }
-}
-
-// Loads a lane's segment (32 consecutive values) from the padded buffer.
-__device__ __forceinline__ void load_seg(const uint32_t* zb, uint32_t seg, uint32_t (&z)[32]) {
-  const uint4* sp = reinterpret_cast<const uint4*>(zb + kSegWords * seg);
-#pragma unroll
-  for (uint32_t c = 0; c < 8; c++) {
-    const uint4 v = sp[c];
-    z[4 * c] = v.x; z[4 * c + 1] = v.y; z[4 * c + 2] = v.z; z[4 * c + 3] = v.w;
+// Delta, ZigZag and column counts of a step: the lanes' segments zs, the first
+// of which continues pred_step (updated to the step's last residual). fast:
+// every delta is below 2^30 in magnitude (zigzag_small). st: stage switches.
+template <bool STAGED>
+__device__ __forceinline__ void step_planes(uint32_t* zs, uint32_t& pred_step, bool fast, uint32_t st, uint32_t (&P)[6]) {
+  const uint32_t last = zs[31];
+  uint32_t pred = __shfl_up_sync(kFull, last, 1);
+  if (lane_id() == 0) pred = pred_step;
+  pred_step = __shfl_sync(kFull, last, 31);
+  if (fast && !(STAGED && (st & (kStageNoDelta | kStageNoZigzag)))) {
+    seg_planes<true>(zs, pred, P);
+  } else {
+    seg_delta_any(zs, pred, st);
+    seg_planes<false>(zs, 0u, P);
   }
 }
 
 // Bytes of the blocks of a row's n residuals (trial pricing, Sec. III-E):
 // header + body bytes summed over the blocks, delta chained from carry.
-__device__ __forceinline__ uint32_t price_row(const uint32_t* zb, uint32_t n, uint32_t carry, uint32_t st) {
+__device__ __forceinline__ uint32_t price_row(uint32_t* zb, uint32_t n, uint32_t carry, bool fast, uint32_t st) {
   const uint32_t lane = lane_id(), j = lane & 3u;
   uint32_t pred_step = carry;
   uint32_t total = 0;
+#pragma unroll 1
   for (uint32_t s0 = 0; s0 < n; s0 += kStepVal) {
     const uint32_t seg = (s0 >> 5) + lane;
-    uint32_t z[32];
-    load_seg(zb, seg, z);
-    uint32_t pred = __shfl_up_sync(kFull, z[31], 1);
-    if (lane == 0) pred = pred_step;
-    pred_step = __shfl_sync(kFull, z[31], 31);
-    delta_zigzag<true, false>(z, pred, st);
+    uint32_t* zs = zb + kSegWords * seg;
+    uint32_t P[6];
+    step_planes<true>(zs, pred_step, fast, st, P);
     const uint32_t g = seg >> 2;
     const uint32_t m = n > 128u * g ? min(128u, n - 128u * g) : 0u;
     uint32_t wmax;
-    const uint32_t key = block_width(z, j, m, wmax);
+    const uint32_t key = block_width(P, j, m, wmax);
     if (m && j == 0) total += 4u + (key >> 14);
   }
   return __reduce_add_sync(kFull, total);
@@ -451,46 +433,57 @@ __device__ __forceinline__ uint32_t price_row(const uint32_t* zb, uint32_t n, ui
 // Low bits of a lane's 32 values (Sec. II, PFOR: value i at bit i b of the
 // block's bit stream, LSB first). 32 values of b bits are exactly b words,
 // so a lane owns words [j b, j b + b) of its block. Words k >= lim are not
-// stored (the lane's share past the block's last value). Values wider than
-// b are cut (masked) when the block has exceptions. Each word is assembled
-// in a 64-bit accumulator (multiply-adds place the bits) and stored once.
+// stored (the lane's share past the block's last value). Each word is
+// assembled in a 64-bit accumulator (multiply-adds place the bits) and stored
+// once: four values at a time where every block of the step has at most 8
+// bits, two up to 16, else one. ANYX: some block of the step has exceptions:
+// values are cut to b bits, and those wider than b come back as a bit mask
+// (of blocks without exceptions: 0).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void pack_low(const uint32_t (&z)[32], const uint32_t* zseg, uint32_t b, uint32_t lim,
-                                         bool masked, uint32_t* wp) {
+template <bool ANYX>
+__device__ __forceinline__ uint32_t pack_low(const uint32_t* zseg, uint32_t b, uint32_t lim, uint32_t* wp) {
+  const uint4* sp = reinterpret_cast<const uint4*>(zseg);
   unsigned long long acc = 0;
-  uint32_t nbit = 0, k = 0;
-  if (__all_sync(kFull, b <= 8u)) {
-    // quads: 4 values = 4b <= 32 bits, at most one word completes per quad
-    const uint32_t bm = (1u << b) - 1u, m1 = 1u << b, u4 = 4u * b;
-    const bool anym = __any_sync(kFull, masked);
-#pragma unroll
-    for (int q = 0; q < 8; q++) {
-      uint32_t a0 = z[4 * q], a1 = z[4 * q + 1], a2 = z[4 * q + 2], a3 = z[4 * q + 3];
-      if (anym) { a0 &= bm; a1 &= bm; a2 &= bm; a3 &= bm; }
-      const uint32_t x = ((a3 * m1 + a2) * m1 + a1) * m1 + a0;
-      acc += (unsigned long long)x * (1u << nbit);
-      nbit += u4;
-      if (nbit >= 32u) {
-        if (k < lim) wp[k] = (uint32_t)acc;
-        k++;
-        acc >>= 32;
-        nbit -= 32u;
+  uint32_t nbit = 0, k = 0, xm = 0;
+  auto put = [&](uint32_t x, uint32_t bits) {  // bits <= 32
+    acc += (unsigned long long)x * (1u << nbit);
+    nbit += bits;
+    if (nbit >= 32u) {
+      if (k < lim) wp[k] = (uint32_t)acc;
+      k++;
+      acc >>= 32;
+      nbit -= 32u;
+    }
+  };
+  if (__all_sync(kFull, b <= 16u)) {
+    const uint32_t bm = (1u << b) - 1u, m1 = 1u << b;
+    const bool quads = __all_sync(kFull, b <= 8u);
+#pragma unroll 2
+    for (uint32_t q = 0; q < 8; q++) {
+      const uint4 v = sp[q];
+      uint32_t a0 = v.x, a1 = v.y, a2 = v.z, a3 = v.w;
+      if (ANYX) {
+        xm |= (min(a0 >> b, 1u) + 2u * min(a1 >> b, 1u) + 4u * min(a2 >> b, 1u) + 8u * min(a3 >> b, 1u)) << (4u * q);
+        a0 &= bm; a1 &= bm; a2 &= bm; a3 &= bm;
+      }
+      const uint32_t lo = a1 * m1 + a0, hi = a3 * m1 + a2;
+      if (quads) {
+        put(hi * (m1 * m1) + lo, 4u * b);
+      } else {
+        put(lo, 2u * b);
+        put(hi, 2u * b);
       }
     }
-  } else {  // some block of the step is wider than 8 bits (rare): one value at a time, rolled
+  } else {  // (a shift by 32 or more gives 0 here: e > 0 implies b < 32)
     const uint32_t bm = b >= 32u ? 0xffffffffu : ((1u << b) - 1u);
 #pragma unroll 1
     for (uint32_t i = 0; i < 32; i++) {
-      acc += (unsigned long long)(zseg[i] & bm) * (1u << nbit);
-      nbit += b;
-      if (nbit >= 32u) {
-        if (k < lim) wp[k] = (uint32_t)acc;
-        k++;
-        acc >>= 32;
-        nbit -= 32u;
-      }
+      const uint32_t v = zseg[i];
+      if (ANYX) xm |= (v & ~bm ? 1u : 0u) << i;
+      put(v & bm, b);
     }
   }
+  return xm;
 }
 
 // ---------------------------------------------------------------------------
@@ -502,16 +495,11 @@ __device__ __forceinline__ void pack_low(const uint32_t (&z)[32], const uint32_t
 // its run of bits [r0 hb, (r0 + c) hb). Words inside a run are stored by its
 // lane; a word where runs meet belongs to the lane whose run holds its first
 // bit, which ORs in the later lanes' leading bits (shuffles) and stores it.
-// zseg: the lane's 32 ZigZag values in shared memory (dynamic indexing).
+// xm: which of the lane's 32 values (zseg) are exceptions (0 for e = 0).
 // Warp-wide (shuffles).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void pack_exceptions(const uint32_t (&z)[32], const uint32_t* zseg, uint32_t j, uint32_t b,
+__device__ __forceinline__ void pack_exceptions(uint32_t xm, const uint32_t* zseg, uint32_t j, uint32_t b,
                                                 uint32_t e, uint32_t hb, uint8_t* blk, uint32_t low_words) {
-  uint32_t xm = 0;
-  if (e) {  // e > 0 implies b < 32
-#pragma unroll
-    for (int i = 0; i < 32; i++) xm |= (z[i] >> b ? 1u : 0u) << i;
-  }
   const uint32_t c = __popc(xm);
   uint32_t incl = c;
   {
@@ -574,32 +562,13 @@ __device__ __forceinline__ uint32_t code_step(uint32_t* zb, uint32_t s0, uint32_
                                               uint32_t st, uint32_t* hdr, uint8_t* body, uint32_t boff) {
   const uint32_t lane = lane_id(), j = lane & 3u;
   const uint32_t seg = (s0 >> 5) + lane;
-  uint32_t z[32];
-  load_seg(zb, seg, z);
-  uint32_t pred = __shfl_up_sync(kFull, z[31], 1);
-  if (lane == 0) pred = pred_step;
-  pred_step = __shfl_sync(kFull, z[31], 31);
-  uint4* sp = reinterpret_cast<uint4*>(zb + kSegWords * seg);  // ZigZag values back, for the exceptions
-  if (!STAGED && fast) {
-    delta_zigzag<false, true>(z, pred, st);
-#pragma unroll
-    for (uint32_t c = 0; c < 8; c++) sp[c] = make_uint4(z[4 * c], z[4 * c + 1], z[4 * c + 2], z[4 * c + 3]);
-  } else {  // deltas of 2^30 or more, or ablated codecs (Sec. IV-H; rare): rolled, through shared memory
-    uint32_t* zs = zb + kSegWords * seg;
-    uint32_t prev = pred;
-#pragma unroll 1
-    for (uint32_t i = 0; i < 32; i++) {
-      const uint32_t e = zs[i];
-      const uint32_t d = (STAGED && (st & kStageNoDelta)) ? e : e - prev;
-      zs[i] = (STAGED && (st & kStageNoZigzag)) ? d : zigzag(d);
-      prev = e;
-    }
-    load_seg(zb, seg, z);
-  }
+  uint32_t* zs = zb + kSegWords * seg;
+  uint32_t P[6];
+  step_planes<STAGED>(zs, pred_step, fast, st, P);
   const uint32_t g = seg >> 2;
   const uint32_t m = n > 128u * g ? min(128u, n - 128u * g) : 0u;
   uint32_t wmax;
-  const uint32_t key = block_width(z, j, m, wmax);
+  const uint32_t key = block_width(P, j, m, wmax);
   const uint32_t b = m ? (key >> 8) & 63u : 0u, e = m ? key & 255u : 0u, f = m ? key >> 14 : 0u;
   const uint32_t hb = e ? wmax - b : 0u;
   // the block's body offset: prefix of the sizes over the step's blocks
@@ -610,8 +579,13 @@ __device__ __forceinline__ uint32_t code_step(uint32_t* zb, uint32_t s0, uint32_
   const uint32_t low_words = (m * b + 31u) >> 5;
   const uint32_t lim = min(b, low_words > j * b ? low_words - j * b : 0u);
   uint8_t* blk = body + off;
-  pack_low(z, zb + kSegWords * seg, b, lim, e != 0u, reinterpret_cast<uint32_t*>(blk) + j * b);
-  if (__any_sync(kFull, e != 0u)) pack_exceptions(z, zb + kSegWords * seg, j, b, e, hb, blk, low_words);
+  uint32_t* wp = reinterpret_cast<uint32_t*>(blk) + j * b;
+  if (__any_sync(kFull, e != 0u)) {
+    const uint32_t xm = pack_low<true>(zs, b, lim, wp);
+    pack_exceptions(xm, zs, j, b, e, hb, blk, low_words);
+  } else {
+    pack_low<false>(zs, b, lim, wp);
+  }
   return tot;
 }
 
@@ -673,15 +647,15 @@ __global__ void __launch_bounds__(32) k_trial(EncParams p) {
   }
   const uint8_t* c1 = cur + test_row(ti) * rowb;
   const uint8_t* p1 = prv + test_row(ti) * rowb;
-  uint32_t n;
+  uint32_t n, qhi;
   const uint32_t kz = all ? 0u : 0xffu;
-  if (at.qkind == 0) n = pass_a_trial<0>(c1, p1, at, W, kz, pmode, zb);
-  else if (at.qkind == 1) n = pass_a_trial<1>(c1, p1, at, W, kz, pmode, zb);
-  else n = pass_a_trial<2>(c1, p1, at, W, kz, pmode, zb);
+  n = pass_a(c1, pmode ? p1 : nullptr, at, W, kz, zb, reinterpret_cast<uint8_t*>(zb + zbuf_words(W)), qhi);
   __syncwarp();
   const bool nd = (st & kStageNoDelta) != 0u;
   if (n) fill_tail(zb, n, nd ? 0u : zb[zaddr(n - 1)]);
-  const uint32_t cost = price_row(zb, n, pmode ? cp : ci, st);
+  // every delta below 2^30 in magnitude: quantized samples and carry below 2^29
+  const uint32_t carry = pmode ? cp : ci;
+  const uint32_t cost = price_row(zb, n, carry, qhi < (1u << 29) && carry + (1u << 29) < (1u << 30), st);
   if (lane_id() == 0) atomicAdd(p.cost + 2 * gs + (pmode ? 1u : 0u), cost);
 }
 
@@ -814,12 +788,14 @@ __device__ __forceinline__ void encode_item(const EncParams& p, const uint32_t k
   const uint32_t* mbw = reinterpret_cast<const uint32_t*>(w.mb);
   const uint32_t below = (1u << lane) - 1u;
   uint32_t nlit = 0;
+#pragma unroll 1
   for (uint32_t jb = 0; jb < nw; jb += 32) {
     const uint32_t jw = jb + lane;
     const bool lit = jw < nw && mask_class(mbw[jw], valid_bits(W, nw, jw)) == 2u;
     nlit += __popc(__ballot_sync(kFull, lit));
   }
   uint32_t litbase = 0;
+#pragma unroll 1
   for (uint32_t jb = 0; jb < nw; jb += 32) {
     const uint32_t jw = jb + lane;
     const uint32_t c = jw < nw ? mbw[jw] : 0u;
@@ -842,6 +818,7 @@ __device__ __forceinline__ void encode_item(const EncParams& p, const uint32_t k
   // 4-byte ones when the quantized samples and the carry stay below 2^29
   const bool fast = at.s <= 2u || (qhi < (1u << 29) && carry + (1u << 29) < (1u << 30));
   uint32_t body_bytes = 0, pred = carry;
+#pragma unroll 1
   for (uint32_t s0 = 0; s0 < n; s0 += kStepVal)
     body_bytes += code_step<STAGED>(w.zb, s0, n, pred, fast, st, hdr, body, body_bytes);
   if (lane == 0) {
@@ -1110,7 +1087,7 @@ int encode_rows_launch(const EncParams& p, RowsLaunch* out) {
   return 0;
 }
 
-size_t trial_smem_bytes_host(uint32_t W) { return 4ull * zbuf_words(W); }
+size_t trial_smem_bytes_host(uint32_t W) { return 4ull * (zbuf_words(W) + ceil_div_u32(W, 32)); }
 
 int launch_encode(const EncParams& p, void* stream, void* const* ev) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
