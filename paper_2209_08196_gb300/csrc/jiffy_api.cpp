@@ -806,6 +806,9 @@ jiffy_status enqueue_encode(Workspace& ws, std::vector<EncJob>& jobs, cudaStream
   p.sec_bytes = reinterpret_cast<unsigned long long*>(d + o_secb);
   p.sec_nnz = reinterpret_cast<uint32_t*>(d + o_secn);
   p.ticket = reinterpret_cast<uint32_t*>(d + o_tick);
+  // up to 1024 rows (4 a thread) the placement kernel sums the sections'
+  // sizes itself, one launch less (a scan of 64 x 1024: 57 -> 54 us a call)
+  p.sum_rows = (items <= 1024 && !zmax_blk) ? 1u : 0u;
   p.staged = staged | (withhold ? 1u : 0u);
   p.withhold = withhold;
   if (zmax_blk) {

@@ -854,7 +854,8 @@ __global__ void __launch_bounds__(WPC * 32, 24 / WPC) k_encode(EncParams p) {
 
 // ----------------------------------------------------------------------------
 // k_sec_sizes: one CTA per section (scan t, attribute a): its bytes (row
-// table + row chunks) and nonzero count.
+// table + row chunks) and nonzero count (larger calls; adding them up in
+// k_encode, two atomics a row, made that 20 us longer where this takes 4).
 // k_place: one CTA per section: the section's offset in the stream (sum over
 // the segment's earlier sections), its row table (end offsets + carries),
 // the copy of each row chunk from its slot and, for attribute 0, the frame
@@ -927,10 +928,37 @@ __global__ void __launch_bounds__(kThreads) k_place(EncParams p) {
   const unsigned long long cap = sg.cap;
   // bytes of the segment's earlier sections: of earlier frames (frame_before)
   // and of this frame's earlier attributes
+  // (small calls: summed from the rows by every CTA, without k_sec_sizes;
+  // their sections are smaller than 2^32 / 64)
+  __shared__ uint32_t s_bytes[kMaxAttr], s_nnz[kMaxAttr];  // this frame's sections
   unsigned long long frame_before = 0, attr_before = 0;
-  for (uint32_t i = threadIdx.x; i < ta; i += kThreads) {
-    if (i < t * A) frame_before += p.sec_bytes[sg.sec_base + i];
-    else attr_before += p.sec_bytes[sg.sec_base + i];
+  if (p.sum_rows) {
+    for (uint32_t i = threadIdx.x; i < A; i += kThreads) {
+      s_bytes[i] = 8u * H;
+      s_nnz[i] = 0u;
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < A * sg.T * H; i += kThreads) {
+      const uint32_t aa = i / (sg.T * H), tt = i / H % sg.T, bytes = p.row_bytes[sg.item_base + i];
+      if (tt < t) {
+        frame_before += bytes;
+      } else if (tt == t) {
+        atomicAdd(s_bytes + aa, bytes);
+        atomicAdd(s_nnz + aa, p.row_nnz[sg.item_base + i]);
+      }
+    }
+    if (threadIdx.x == 0) frame_before += 8ull * H * t * A;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < a; i += kThreads) attr_before += s_bytes[i];
+  } else {
+    for (uint32_t i = threadIdx.x; i < ta; i += kThreads) {
+      if (i < t * A) frame_before += p.sec_bytes[sg.sec_base + i];
+      else attr_before += p.sec_bytes[sg.sec_base + i];
+    }
+    for (uint32_t i = threadIdx.x; i < A; i += kThreads) {
+      s_bytes[i] = (uint32_t)p.sec_bytes[sg.sec_base + t * A + i];
+      s_nnz[i] = p.sec_nnz[sg.sec_base + t * A + i];
+    }
   }
   frame_before = cta_sum_u64(frame_before, s_red);
   attr_before = cta_sum_u64(attr_before, s_red);
@@ -1023,14 +1051,14 @@ __global__ void __launch_bounds__(kThreads) k_place(EncParams p) {
   if (part == 0 && a == 0 && threadIdx.x == 0) {
     const uint32_t f0 = sg.sec_base + t * A;
     unsigned long long fbytes = sg.fhdr;
-    for (uint32_t aa = 0; aa < A; aa++) fbytes += p.sec_bytes[f0 + aa];
+    for (uint32_t aa = 0; aa < A; aa++) fbytes += s_bytes[aa];
     put_u32_guarded(out, cap, frame_at, (uint32_t)fbytes, sg.err);
     put_u32_guarded(out, cap, frame_at + 4, sg.frame0 + t, sg.err);
     for (uint32_t aa = 0; aa < A; aa++) {
       const unsigned long long h = frame_at + 8ull + 12ull * aa;
       put_u32_guarded(out, cap, h, p.modes[f0 + aa], sg.err);
-      put_u32_guarded(out, cap, h + 4, (uint32_t)p.sec_bytes[f0 + aa], sg.err);
-      put_u32_guarded(out, cap, h + 8, p.sec_nnz[f0 + aa], sg.err);
+      put_u32_guarded(out, cap, h + 4, s_bytes[aa], sg.err);
+      put_u32_guarded(out, cap, h + 8, s_nnz[aa], sg.err);
     }
     sg.frame_off[t] = frame_at;
     if (t + 1 == sg.T) sg.frame_off[sg.T] = frame_at + fbytes;
@@ -1136,7 +1164,7 @@ int launch_encode(const EncParams& p, void* stream, void* const* ev) {
   mark(2);
   rc = launch_zstd_encode(p, st);
   if (rc != 0) return rc;
-  k_sec_sizes<<<p.n_sec, kThreads, 0, st>>>(p);
+  if (!p.sum_rows) k_sec_sizes<<<p.n_sec, kThreads, 0, st>>>(p);
   k_place<<<p.n_sec * kPlaceSplit, kThreads, s_place, st>>>(p);
   mark(3);
   return (int)cudaGetLastError();

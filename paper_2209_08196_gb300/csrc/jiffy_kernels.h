@@ -63,6 +63,7 @@ struct EncParams {
   uint8_t* slots;                // packed row chunks, slot_base + local item * slot_bytes
   unsigned long long* sec_bytes; // [n_sec] section bytes (row table + chunks)
   uint32_t* sec_nnz;             // [n_sec]
+  uint32_t sum_rows;             // 1: a small call, the placement kernel adds the sections' rows up itself
   uint32_t* ticket;
   uint32_t wpc;                  // rows kernel: warps per CTA (1, 2, 4; 0 = by shared memory)
   uint32_t ctas_per_sm;          // rows kernel: resident CTAs per SM (0 = occupancy limit)
