@@ -60,7 +60,7 @@ STAGE_ZSTD_MASK = 8  # the zero mask as one Zstandard frame per section (Sec. II
 
 
 _L = None
-_ENC_BATCH_ADDR = _DEC_BATCH_ADDR = None
+_BATCH_ADDR = {}  # the batched entry points over plain addresses
 
 
 def _lib() -> ctypes.CDLL:
@@ -125,10 +125,10 @@ def _lib() -> ctypes.CDLL:
         L.jiffy_decode_batch_async.argtypes = L.jiffy_decode_batch.argtypes
         L.jiffy_batch_wait.restype = ctypes.c_int
         L.jiffy_batch_wait.argtypes = [vp]
-        # the same batched entry points over plain addresses (array-marshalled calls)
-        global _ENC_BATCH_ADDR, _DEC_BATCH_ADDR
-        _ENC_BATCH_ADDR = ctypes.CFUNCTYPE(ctypes.c_int, vp, u32, *([vp] * 9))(("jiffy_encode_batch_async", L))
-        _DEC_BATCH_ADDR = ctypes.CFUNCTYPE(ctypes.c_int, vp, u32, *([vp] * 8))(("jiffy_decode_batch_async", L))
+        # the same batched entry points over plain addresses (arguments marshalled as numpy arrays)
+        for name, n_ptr in (("jiffy_encode_batch", 9), ("jiffy_decode_batch", 8)):
+            for f in (name, name + "_async"):
+                _BATCH_ADDR[f] = ctypes.CFUNCTYPE(ctypes.c_int, vp, u32, *([vp] * n_ptr))((f, L))
         L.jiffy_batch_set_graphs.restype = ctypes.c_int
         L.jiffy_batch_set_graphs.argtypes = [vp, ctypes.c_int]
         L.jiffy_batch_set_autotune.restype = ctypes.c_int
@@ -171,8 +171,8 @@ def _attrs(attrs):
 
 
 def _stream_ptr(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:  # the current stream's handle, without the Stream object
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -511,8 +511,63 @@ def jiffy_stream_device_bytes(h: Handle) -> int:
     return _lib().jiffy_stream_device_bytes(h.ptr)
 
 
-def _addr(a) -> int:
-    return ctypes.cast(a, ctypes.c_void_p).value
+def _batch_tables(handles, planes, what: str):
+    """(scans per stream, plane pointer tables of all streams in one uint64
+    array, where each stream's table starts). Planes are given and checked per
+    stream as for the sequence calls (_seq_ptrs); the pointers of all streams
+    are computed at once (64 streams: a table of their own each took some 5 us
+    a stream)."""
+    counts, bases, steps, per_scan, scans = [], [], [], [], []
+    for h, pl in zip(handles, planes):
+        p0 = pl[0]
+        attrs = h.attrs
+        if isinstance(p0, torch.Tensor) and len(pl) == len(attrs) and p0.dim() == 3:
+            T, HW = p0.shape[0], h.H * h.W
+            for p, (s, _) in zip(pl, attrs):
+                sh = p.shape
+                if sh[0] != T or not p.is_cuda or p.element_size() != s or not p.is_contiguous() or sh[1] * sh[2] != HW:
+                    raise ValueError("%s %d: expected a contiguous CUDA tensor of %d x %d x %d %d-byte samples, got %s %s"
+                                     % (what, len(bases) - sum(per_scan), T, h.H, h.W, s, tuple(sh), p.dtype))
+                bases.append(p.data_ptr())
+                steps.append(HW * s)
+            per_scan.append(len(pl))
+            scans.append(T)
+        else:  # scan by scan: one "scan" of all its planes
+            T, flat = _seq_planes(h, pl)
+            for i, p in enumerate(flat):
+                _check_plane(p, h.H, h.W, attrs[i % len(attrs)][0], "%s %d" % (what, i))
+                bases.append(p.data_ptr())
+                steps.append(0)
+            per_scan.append(len(flat))
+            scans.append(1)
+        counts.append(T)
+    A, T = np.array(per_scan, dtype=np.int64), np.array(scans, dtype=np.int64)
+    n = A * T  # pointers of each stream, scan-major
+    ends = np.cumsum(n)
+    starts = ends - n
+    k = np.arange(int(ends[-1]) if len(n) else 0, dtype=np.int64) - np.repeat(starts, n)
+    t, a = np.divmod(k, np.repeat(A, n))
+    at = np.repeat(np.cumsum(A) - A, n) + a
+    table = np.array(bases, dtype=np.uint64)[at] + (np.array(steps, dtype=np.int64)[at] * t).astype(np.uint64)
+    return counts, table, starts
+
+
+def _offset_starts(counts):
+    n = np.array(counts, dtype=np.int64) + 1
+    return np.cumsum(n) - n
+
+
+def _per_stream(values, n: int, dtype=np.uint64):
+    """One value per stream; missing ones are 0 (the C ABI refuses them)."""
+    if len(values) > n:
+        raise IndexError("more arguments than streams")
+    out = np.zeros(n, dtype=dtype)
+    out[:len(values)] = values
+    return out
+
+
+def _handle_ptrs(handles):
+    return np.array([h.ptr or 0 for h in handles], dtype=np.uint64)
 
 
 class _EncCall:
@@ -520,48 +575,51 @@ class _EncCall:
 
     def __init__(self, handles, planes, outs):
         n = len(handles)
-        flats = [_seq_ptrs(h, pl, "plane") for h, pl in zip(handles, planes)]
+        counts, self.table, starts = _batch_tables(handles, planes, "plane")
         self.n = n
-        self.streams = (ctypes.c_void_p * n)(*[h.ptr for h in handles])
-        self.n_scans = (ctypes.c_uint32 * n)(*[T for T, _ in flats])
-        self.parr = [arr for _, arr in flats]
-        self.planes = (ctypes.c_void_p * n)(*[_addr(a) for a in self.parr])
-        self.outs = (ctypes.c_void_p * n)(*[o.data_ptr() for o in outs])
-        self.caps = (ctypes.c_size_t * n)(*[o.numel() * o.element_size() for o in outs])
-        self.offs = [(ctypes.c_uint64 * (T + 1))() for T, _ in flats]
-        self.offs_pp = (ctypes.c_void_p * n)(*[_addr(a) for a in self.offs])
-        self.lens = (ctypes.c_size_t * n)()
-        self.sts = (ctypes.c_int * n)()
+        self.streams = _handle_ptrs(handles)
+        self.n_scans = _per_stream(counts, n, np.uint32)
+        self.planes = _per_stream(self.table.ctypes.data + 8 * starts, n)
+        self.outs = _per_stream([o.data_ptr() for o in outs], n)
+        self.caps = _per_stream([o.numel() * o.element_size() for o in outs], n)
+        self.ostarts = _offset_starts(counts)
+        self.offs = np.zeros(sum(counts) + n, dtype=np.uint64)
+        self.offs_pp = _per_stream(self.offs.ctypes.data + 8 * self.ostarts, n)
+        self.lens = np.zeros(n, dtype=np.uint64)
+        self.sts = np.zeros(n, dtype=np.int32)
 
     def args(self, b, stream):
-        return (b.ptr, self.n, self.streams, self.n_scans, self.planes, self.outs, self.caps, self.offs_pp,
-                self.lens, self.sts, _stream_ptr(stream))
+        return (b.ptr, self.n, *(x.ctypes.data for x in (self.streams, self.n_scans, self.planes, self.outs, self.caps,
+                                                         self.offs_pp, self.lens, self.sts)), _stream_ptr(stream))
 
     def result(self):
-        return [(self.lens[i], list(self.offs[i])) for i in range(self.n)]
+        offs, lens = self.offs.tolist(), self.lens.tolist()
+        return [(lens[i], offs[o:o + int(c) + 1]) for i, (o, c) in enumerate(zip(self.ostarts.tolist(), self.n_scans))]
 
 
 class _DecCall:
     def __init__(self, handles, bufs, lengths, offsets, planes_out):
         n = len(handles)
-        flats = [_seq_ptrs(h, pl, "output plane") for h, pl in zip(handles, planes_out)]
-        for (T, _), o in zip(flats, offsets):
+        counts, self.table, starts = _batch_tables(handles, planes_out, "output plane")
+        flat, given = [], []
+        for T, o in zip(counts, offsets):
             if len(o) != T + 1:
                 raise ValueError("need T + 1 frame offsets")
+            flat.extend([int(v) for v in o])
+            given.append(T)
         self.n = n
-        self.streams = (ctypes.c_void_p * n)(*[h.ptr for h in handles])
-        self.n_frames = (ctypes.c_uint32 * n)(*[T for T, _ in flats])
-        self.ins = (ctypes.c_void_p * n)(*[x.data_ptr() for x in bufs])
-        self.lens = (ctypes.c_size_t * n)(*[int(x) for x in lengths])
-        self.offs = [(ctypes.c_uint64 * len(o))(*[int(v) for v in o]) for o in offsets]
-        self.offs_pp = (ctypes.c_void_p * n)(*[_addr(a) for a in self.offs])
-        self.parr = [arr for _, arr in flats]
-        self.planes = (ctypes.c_void_p * n)(*[_addr(a) for a in self.parr])
-        self.sts = (ctypes.c_int * n)()
+        self.streams = _handle_ptrs(handles)
+        self.n_frames = _per_stream(counts, n, np.uint32)
+        self.ins = _per_stream([x.data_ptr() for x in bufs], n)
+        self.lens = _per_stream([int(x) for x in lengths], n)
+        self.offs = np.array(flat, dtype=np.uint64)
+        self.offs_pp = _per_stream(self.offs.ctypes.data + 8 * _offset_starts(given), n)
+        self.planes = _per_stream(self.table.ctypes.data + 8 * starts, n)
+        self.sts = np.zeros(n, dtype=np.int32)
 
     def args(self, b, stream):
-        return (b.ptr, self.n, self.streams, self.n_frames, self.ins, self.lens, self.offs_pp, self.planes,
-                self.sts, _stream_ptr(stream))
+        return (b.ptr, self.n, *(x.ctypes.data for x in (self.streams, self.n_frames, self.ins, self.lens, self.offs_pp,
+                                                         self.planes, self.sts)), _stream_ptr(stream))
 
 
 def jiffy_encode_batch(b: Batch, handles, planes, outs, stream=None):
@@ -569,9 +627,10 @@ def jiffy_encode_batch(b: Batch, handles, planes, outs, stream=None):
     into outs[i], all streams in one pass. Returns a list of (bytes, frame
     offsets) per stream."""
     c = _EncCall(handles, planes, outs)
-    st = _lib().jiffy_encode_batch(*c.args(b, stream))
+    _lib()
+    st = _BATCH_ADDR["jiffy_encode_batch"](*c.args(b, stream))
     if st != 0:
-        raise BatchError(st, "jiffy_encode_batch", list(c.sts), required=list(c.lens))
+        raise BatchError(st, "jiffy_encode_batch", c.sts.tolist(), required=c.lens.tolist())
     return c.result()
 
 
@@ -579,26 +638,29 @@ def jiffy_decode_batch(b: Batch, handles, bufs, lengths, offsets, planes_out, st
     """Decodes, per stream i, the frames of bufs[i] (lengths[i] bytes, frame
     offsets offsets[i]) into planes_out[i], all streams in one pass."""
     c = _DecCall(handles, bufs, lengths, offsets, planes_out)
-    st = _lib().jiffy_decode_batch(*c.args(b, stream))
+    _lib()
+    st = _BATCH_ADDR["jiffy_decode_batch"](*c.args(b, stream))
     if st != 0:
-        raise BatchError(st, "jiffy_decode_batch", list(c.sts))
+        raise BatchError(st, "jiffy_decode_batch", c.sts.tolist())
 
 
 def jiffy_encode_batch_async(b: Batch, handles, planes, outs, stream=None):
     """Enqueues a batched encode and returns at once; jiffy_batch_wait(b)
     returns its result (as jiffy_encode_batch does)."""
     c = _EncCall(handles, planes, outs)
-    st = _lib().jiffy_encode_batch_async(*c.args(b, stream))
+    _lib()
+    st = _BATCH_ADDR["jiffy_encode_batch_async"](*c.args(b, stream))
     if st != 0:
-        raise BatchError(st, "jiffy_encode_batch_async", list(c.sts))
+        raise BatchError(st, "jiffy_encode_batch_async", c.sts.tolist())
     b.pending = ("encode", c)
 
 
 def jiffy_decode_batch_async(b: Batch, handles, bufs, lengths, offsets, planes_out, stream=None):
     c = _DecCall(handles, bufs, lengths, offsets, planes_out)
-    st = _lib().jiffy_decode_batch_async(*c.args(b, stream))
+    _lib()
+    st = _BATCH_ADDR["jiffy_decode_batch_async"](*c.args(b, stream))
     if st != 0:
-        raise BatchError(st, "jiffy_decode_batch_async", list(c.sts))
+        raise BatchError(st, "jiffy_decode_batch_async", c.sts.tolist())
     b.pending = ("decode", c)
 
 
@@ -639,7 +701,7 @@ def jiffy_encode_batch_async_arrays(b: Batch, streams, n_scans, plane_tables, ou
     lens = np.zeros(n, dtype=np.uint64)
     sts = np.zeros(n, dtype=np.int32)
     keep = (streams, n_scans, tables, outs, caps, offs_pp)
-    st = _ENC_BATCH_ADDR(b.ptr, n, streams.ctypes.data, n_scans.ctypes.data, tables.ctypes.data, outs.ctypes.data,
+    st = _BATCH_ADDR["jiffy_encode_batch_async"](b.ptr, n, streams.ctypes.data, n_scans.ctypes.data, tables.ctypes.data, outs.ctypes.data,
                          caps.ctypes.data, offs_pp.ctypes.data, lens.ctypes.data, sts.ctypes.data,
                          _stream_ptr(stream))
     if st != 0:
@@ -667,7 +729,7 @@ def jiffy_decode_batch_async_arrays(b: Batch, streams, n_frames, ins, in_lens, o
     offs_pp = _u64(offsets.ctypes.data + 8 * starts)
     sts = np.zeros(n, dtype=np.int32)
     keep = (streams, n_frames, ins, in_lens, offsets, offs_pp, tables)
-    st = _DEC_BATCH_ADDR(b.ptr, n, streams.ctypes.data, n_frames.ctypes.data, ins.ctypes.data, in_lens.ctypes.data,
+    st = _BATCH_ADDR["jiffy_decode_batch_async"](b.ptr, n, streams.ctypes.data, n_frames.ctypes.data, ins.ctypes.data, in_lens.ctypes.data,
                          offs_pp.ctypes.data, tables.ctypes.data, sts.ctypes.data, _stream_ptr(stream))
     if st != 0:
         raise BatchError(st, "jiffy_decode_batch_async", sts.tolist())
@@ -689,10 +751,10 @@ def jiffy_batch_wait(b: Batch):
     st = _lib().jiffy_batch_wait(b.ptr)
     b.pending = None
     if st != 0:
-        sts = c.sts.tolist() if isinstance(c, _ArrayCall) else (list(c.sts) if c else [])
+        sts = c.sts.tolist() if c else []
         req = res = None
         if kind == "encode":
-            req = c.lens.tolist() if isinstance(c, _ArrayCall) else list(c.lens)
+            req = c.lens.tolist()
             res = c.result() if isinstance(c, _ArrayCall) else None
         raise BatchError(st, "jiffy_batch_wait", sts, required=req, result=res)
     return c.result() if kind == "encode" else None
