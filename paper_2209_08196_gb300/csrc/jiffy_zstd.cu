@@ -38,8 +38,8 @@
 //   the block-end index, the frame and block headers, stages a Compressed
 //   block in shared memory, reads the tree (lane 0), builds the decoding
 //   table (warp ballots per weight class) and decodes the streams, one lane
-//   per stream, each through a 64-bit window of its bits held in registers,
-//   into the section's mask bytes; the rows kernel reads its rows from there.
+//   per stream, up to two literals a table lookup, through a 64-bit window of
+//   its bits held in registers, into the section's mask bytes; the rows kernel reads its rows from there.
 //   Anything that is not what the writer can produce sets the segment's
 //   CORRUPT flag.
 #include "jiffy_device.cuh"
@@ -139,6 +139,7 @@ struct ZEnc {
   uint8_t fenc[16][64];           // FSE encoding: (symbol, next state) -> state
   FseTable ft;
   uint32_t fhist[16], fnorm[16], fnext[16];
+  uint32_t fbits[32], fhead;      // FSE-coded weights; bytes of the tree before them
   uint32_t gcnt[8][kZMaxBits + 1];  // symbols of each weight per group of 32 values
   uint32_t wsum[kZW];             // scan scratch
   uint32_t pb[5];                 // literal bits before each stream boundary
@@ -213,27 +214,44 @@ __device__ uint32_t fse_write(ZEnc& z, uint32_t n) {
   const uint32_t head = w.close();
   if (head >= 127u) return 0;
   // two states from the last weight back: weight i is emitted by state i%2;
-  // the fields come out in the order they are written
-  BitPut b{z.tree + 1 + head, 127u - head, 0u, 0ull, 0u};
-  uint32_t st[2] = {0, 0};
-  for (int i = (int)n - 1; i >= 0; i--) {
-    const uint32_t q = (uint32_t)i & 1u, sy = z.weight[i];
-    if (i >= (int)n - 2) {
-      uint32_t u = 0;
-      while (z.ft.sym[u] != sy) u++;
-      st[q] = u;
-      continue;
+  // the fields come out in the order they are written, whole words of them to
+  // z.fbits (the CTA copies them behind the description). The two states are
+  // two independent chains of one table lookup per weight.
+  unsigned long long acc = 0;
+  uint32_t nacc = 0, nw = 0;
+  auto put = [&](uint32_t v, uint32_t nb) {  // nb <= 6
+    acc |= (unsigned long long)(v & ((1u << nb) - 1u)) << nacc;
+    nacc += nb;
+    if (nacc >= 32u) {
+      if (nw < 32u) z.fbits[nw] = (uint32_t)acc;
+      nw++;
+      acc >>= 32;
+      nacc -= 32u;
     }
-    const uint32_t v = st[q], u = z.fenc[sy][v];
-    b.put(v - z.ft.base[u], z.ft.nb[u]);
-    st[q] = u;
+  };
+  auto first = [&](uint32_t sy) {
+    uint32_t u = 0;
+    while (z.ft.sym[u] != sy) u++;
+    return u;
+  };
+  auto step = [&](uint32_t& st, uint32_t sy) {
+    const uint32_t u = z.fenc[sy][st];
+    put(st - z.ft.base[u], z.ft.nb[u]);
+    st = u;
+  };
+  uint32_t sa = first(z.weight[n - 1u]), sb = first(z.weight[n - 2u]);
+  for (int i = (int)n - 3; i >= 0; i -= 2) {
+    step(sa, z.weight[i]);
+    if (i > 0) step(sb, z.weight[i - 1]);
   }
-  b.put(st[1], kZFseLog);
-  b.put(st[0], kZFseLog);
-  b.put(1u, 1u);
-  const uint32_t body = b.close();
+  put((n - 1u) & 1u ? sa : sb, kZFseLog);  // the odd weights' state, then the even ones'
+  put((n - 1u) & 1u ? sb : sa, kZFseLog);
+  put(1u, 1u);
+  const uint32_t body = 4u * nw + (nacc + 7u) / 8u;
+  if (nw < 32u) z.fbits[nw] = (uint32_t)acc;
   if (head + body >= 128u) return 0;
   z.tree[0] = (uint8_t)(head + body);
+  z.fhead = 1u + head;
   return 1u + head + body;
 }
 
@@ -344,8 +362,8 @@ __global__ void __launch_bounds__(kZT, 8) k_zstd_enc(EncParams p) {
   __syncthreads();
 
   // ---- code lengths: the present symbols sorted by (count, value) (a
-  //      bitonic sort of count << 8 | value), merged on thread 0 with the
-  //      queue heads in registers, internal depths top-down; each leaf's
+  //      bitonic sort of count << 8 | value), merged on thread 0,
+  //      depths of the internal nodes by pointer doubling; each leaf's
   //      length is its parent's depth + 1. Counts halved while too deep.
   for (;;) {
     uint32_t c2[2];
@@ -359,33 +377,75 @@ __global__ void __launch_bounds__(kZT, 8) k_zstd_enc(EncParams p) {
     const uint32_t nsym = (uint32_t)__syncthreads_count(c2[0] != 0u) + (uint32_t)__syncthreads_count(c2[1] != 0u);
     bitonic256(z.key);
     if (tid == 0) {
-      uint32_t lf = 0, nd = nsym, next = nsym;
-      uint32_t lw = z.key[0] >> 8, ndw = 0;
+      // two-queue merge. The first two weights of each queue decide a step;
+      // they and the two behind them are held in registers (~0: none), so a
+      // step's chain is its comparisons and not the loads: the loads fill the
+      // third and fourth places, needed a step later at the earliest
+      constexpr uint32_t kNone = 0xffffffffu;
+      uint32_t lf = 0, nd = nsym, next = nsym;  // queue heads; the next node
+      auto leaf = [&](uint32_t i) { return i < nsym ? z.key[i] >> 8 : kNone; };
+      auto node = [&](uint32_t i) { return i < next ? z.wnode[i] : kNone; };
+      uint32_t l0 = leaf(0), l1 = leaf(1), l2 = leaf(2), l3 = leaf(3);
+      uint32_t n0 = kNone, n1 = kNone, n2 = kNone, n3 = kNone;
       for (uint32_t k = 0; k + 1 < nsym; k++) {
-        uint32_t pk[2], pw[2];
+        const bool a = l0 <= n0;                    // first: a leaf? (ties take it)
+        const bool b = (a ? l1 : l0) <= (a ? n0 : n1);  // second
+        const uint32_t w0 = a ? l0 : n0, w1 = a ? (b ? l1 : n0) : (b ? l0 : n1);
+        const uint32_t from_l = (a ? 1u : 0u) + (b ? 1u : 0u);
+        const uint32_t p0 = a ? lf : nd, p1 = a ? (b ? lf + 1u : nd) : (b ? lf : nd + 1u);
+        const uint32_t ws = w0 + w1;
+        z.parent[p0] = (uint16_t)next;
+        z.parent[p1] = (uint16_t)next;
+        z.wnode[next] = ws;
+        next++;
+        lf += from_l;
+        nd += 2u - from_l;
+        l0 = from_l == 0u ? l0 : from_l == 1u ? l1 : l2;
+        l1 = from_l == 0u ? l1 : from_l == 1u ? l2 : l3;
+        n0 = from_l == 2u ? n0 : from_l == 1u ? n1 : n2;
+        n1 = from_l == 2u ? n1 : from_l == 1u ? n2 : n3;
+        const uint32_t left = next - nd;  // nodes queued, the new one last
+        n0 = left == 1u ? ws : n0;
+        n1 = left == 2u ? ws : n1;
+        l2 = leaf(lf + 2u);
+        l3 = leaf(lf + 3u);
+        n2 = node(nd + 2u);
+        n3 = node(nd + 3u);
+      }
+    }
+    __syncthreads();
+    // depths of the internal nodes (root last) by pointer doubling
+    {
+      const uint32_t root = 2u * nsym - 2u;
+      uint32_t dep[2], par[2];
 #pragma unroll
-        for (uint32_t q = 0; q < 2; q++) {
-          if (lf < nsym && (nd >= next || lw <= ndw)) {
-            pk[q] = lf;
-            pw[q] = lw;
-            lf++;
-            lw = lf < nsym ? (z.key[lf] >> 8) : 0u;
-          } else {
-            pk[q] = nd;
-            pw[q] = ndw;
-            nd++;
-            ndw = nd < next ? z.wnode[nd] : 0u;
+      for (uint32_t h = 0; h < 2; h++) {
+        const uint32_t i = nsym + tid + kZT * h;
+        dep[h] = i < root ? 1u : 0u;
+        par[h] = i < root ? z.parent[i] : root;
+        if (i <= root) z.depth[i] = (uint8_t)dep[h];
+        if (i == root) z.parent[i] = (uint16_t)root;
+      }
+      __syncthreads();
+      while (__syncthreads_or((par[0] != root) | (par[1] != root))) {
+        uint32_t d2[2], p2[2];
+#pragma unroll
+        for (uint32_t h = 0; h < 2; h++) {
+          d2[h] = z.depth[par[h]];
+          p2[h] = z.parent[par[h]];
+        }
+        __syncthreads();
+#pragma unroll
+        for (uint32_t h = 0; h < 2; h++) {
+          const uint32_t i = nsym + tid + kZT * h;
+          dep[h] += d2[h];
+          par[h] = p2[h];
+          if (i < root) {
+            z.depth[i] = (uint8_t)dep[h];
+            z.parent[i] = (uint16_t)par[h];
           }
         }
-        const uint32_t ws = pw[0] + pw[1];
-        z.wnode[next] = ws;
-        z.parent[pk[0]] = (uint16_t)next;
-        z.parent[pk[1]] = (uint16_t)next;
-        if (nd == next) ndw = ws;  // the node queue was empty: the new node heads it
-        next++;
       }
-      z.depth[next - 1] = 0;
-      for (int i = (int)next - 2; i >= (int)nsym; i--) z.depth[i] = (uint8_t)(z.depth[z.parent[i]] + 1u);
     }
     __syncthreads();
     for (uint32_t i = tid; i < nsym; i += kZT) {
@@ -458,6 +518,8 @@ __global__ void __launch_bounds__(kZT, 8) k_zstd_enc(EncParams p) {
     if (z.fok && tid < 64u) fse_fill(z, tid);
     __syncthreads();
     if (tid == 0) z.tree_len = z.fok ? fse_write(z, last) : 0u;
+    __syncthreads();
+    if (z.tree_len && z.fhead + tid < z.tree_len) z.tree[z.fhead + tid] = reinterpret_cast<const uint8_t*>(z.fbits)[tid];
   }
 
   // ---- literal bit counts: per-thread sums, CTA scan, stream boundaries
@@ -560,7 +622,9 @@ constexpr uint32_t kBlkWords = (kZBlock + 128) / 4;  // a block's content (<= 81
 
 struct ZDec {
   uint32_t blkw[kBlkWords];   // a Compressed block's content (from byte blk_at), zero slack for the peeks
-  uint16_t dt[1u << kZMaxBits];  // decoding table: symbol | code bits << 8
+  // decoding table: symbol | code bits << 8, and where a second code fits
+  // into the index: second symbol << 16 | bits of both << 24 (else 0)
+  uint32_t dt[1u << kZMaxBits];
   uint8_t weight[256];
   uint8_t sorted[256];        // symbols with a weight, by (weight, value)
   uint32_t cls_base[kZMaxBits + 1], cls_pos[kZMaxBits + 1], cls_cnt[kZMaxBits + 1];
@@ -703,46 +767,67 @@ __device__ bool tree_weights(ZDec& z, uint32_t lane) {
   return true;
 }
 
-// One stream of cnt literals (lanes 0..3); false if malformed. The bits
-// below the read position sit in a 64-bit window (bits [bot, bot + k) of the
-// stream in its low k bits); whenever fewer than 32 remain it takes the 32
-// bits below it (bytes before the stream's start read as zero), then two
-// literals are decoded. The stream is well formed if the last literal ends
-// exactly at bit 0. Loads and refills are predicated, so the lanes of
-// different streams do not diverge.
-__device__ bool read_stream(const ZDec& z, const uint8_t* s, uint32_t len, uint8_t* out, uint32_t cnt) {
-  if (len == 0 || s[len - 1] == 0) return false;
-  const int p0 = (int)(8u * (len - 1u) + hibit(s[len - 1]));
-  const uint32_t mb = z.maxbits, mask = (1u << mb) - 1u;
-  int bot = p0 & ~7;
-  unsigned long long win = s[bot >> 3] & ((1u << (p0 - bot)) - 1u);
-  int k = p0 - bot;
-  auto refill = [&]() {
-    const int b = (bot >> 3) - 4;
-    uint32_t w = 0;
+// One stream of cnt literals (the lanes of `lanes` together, one each); false
+// if malformed. s: its bytes in z.blkw. The next bits stand at the top of a
+// 64-bit window hi:lo, `have` of them unread (at least 32 after a refill);
+// the word below it is loaded a refill ahead, so the chain from literal to
+// literal is a shift, a table lookup and a shift. A lookup gives two literals
+// where both codes fit into the index (mask bytes take 3 to 4 bits, so nearly
+// always). Lanes that are done go on without storing: everything is
+// predicated, so that the lanes stay together. Bits below the stream's start
+// read as whatever lies there: the stream is well formed if the last literal
+// ends exactly at its first bit.
+__device__ bool read_stream(const ZDec& z, const uint8_t* s, uint32_t len, uint8_t* out, uint32_t cnt, uint32_t lanes) {
+  const bool ok = len != 0u && s[len - 1] != 0;
+  const int start = 8 * (int)(s - reinterpret_cast<const uint8_t*>(z.blkw));
+  const int p = ok ? start + (int)(8u * (len - 1u) + hibit(s[len - 1])) : start;
+  if (!ok) cnt = 0;
+  const uint32_t down = 32u - z.maxbits;
+  auto word = [&](int w) { return z.blkw[max(w, 0)]; };  // (below the block: never part of a well-formed stream)
+  int wi = (p >> 5) - 1;  // the lower word of the window
+  uint32_t have = (uint32_t)(p - 32 * wi);  // 32 .. 63
+  uint32_t hi = __funnelshift_l(word(wi), word(wi + 1), 64u - have), lo = word(wi) << ((64u - have) & 31u);
+  if (have == 32u) {  // (a shift by a whole word)
+    hi = word(wi);
+    lo = 0u;
+  }
+  uint32_t next = word(wi - 1), i = 0;
+  int left = p - start;  // unread bits of the stream
+  auto take = [&](uint32_t n) {
+    hi = __funnelshift_l(lo, hi, n);
+    lo <<= n;
+    have -= n;
+    left -= (int)n;
+  };
+  auto refill = [&]() {  // have >= 10
+    const bool need = have < 32u;
+    hi |= need ? next >> have : 0u;
+    lo = need ? next << (32u - have) : lo;
+    have += need ? 32u : 0u;
+    wi -= need ? 1 : 0;
+    next = word(wi - 1);
+  };
+  while (__any_sync(lanes, i + 3u < cnt)) {
+    refill();
 #pragma unroll
-    for (int q = 0; q < 4; q++) w |= (b + q >= 0 ? (uint32_t)s[b + q] : 0u) << (8 * q);
-    const bool need = k < 32;
-    win = need ? (win << 32) | w : win;
-    bot = need ? bot - 32 : bot;
-    k = need ? k + 32 : k;
-  };
-  auto one = [&](uint32_t i) {
-    const uint32_t e = z.dt[(uint32_t)(win >> (k - (int)mb)) & mask];
-    out[i] = (uint8_t)e;
-    k -= (int)(e >> 8);
-  };
-  uint32_t i = 0;
-  for (; i + 1u < cnt; i += 2u) {
-    refill();
-    one(i);
-    one(i + 1u);
+    for (int q = 0; q < 2; q++) {
+      const uint32_t e = z.dt[hi >> down];
+      const bool on = i + 1u < cnt, two = on && (e >> 24);
+      if (on) out[i] = (uint8_t)e;
+      if (two) out[i + 1u] = (uint8_t)(e >> 16);
+      i += two ? 2u : (on ? 1u : 0u);
+      take(two ? e >> 24 : (on ? (e >> 8) & 0xffu : 0u));
+    }
   }
-  if (i < cnt) {
+  while (__any_sync(lanes, i < cnt)) {
     refill();
-    one(i);
+    const uint32_t e = z.dt[hi >> down];
+    const bool on = i < cnt;
+    if (on) out[i] = (uint8_t)e;
+    i += on ? 1u : 0u;
+    take(on ? (e >> 8) & 0xffu : 0u);
   }
-  return bot + k == 0;
+  return ok && left == 0;
 }
 
 __global__ void __launch_bounds__(32) k_zstd_dec(DecParams p) {
@@ -873,7 +958,14 @@ __global__ void __launch_bounds__(32) k_zstd_dec(DecParams p) {
   for (uint32_t w = 1; w <= mb; w++) {
     const uint32_t sh = w - 1u, total = z.cls_cnt[w] << sh, b = z.cls_base[w], p0 = z.cls_pos[w];
     const uint32_t lenbits = (mb + 1u - w) << 8;
-    for (uint32_t e = lane; e < total; e += 32u) z.dt[b + e] = (uint16_t)(z.sorted[p0 + (e >> sh)] | lenbits);
+    for (uint32_t e = lane; e < total; e += 32u) z.dt[b + e] = z.sorted[p0 + (e >> sh)] | lenbits;
+  }
+  __syncwarp();
+  // the second literal of each index (a lane changes only the upper halves)
+  for (uint32_t e = lane; e < (1u << mb); e += 32u) {
+    const uint32_t l1 = (z.dt[e] >> 8) & 0xffu, s2 = z.dt[(e << l1) & ((1u << mb) - 1u)];
+    const uint32_t both = l1 + ((s2 >> 8) & 0xffu);
+    if (both <= mb) reinterpret_cast<uint16_t*>(&z.dt[e])[1] = (uint16_t)((s2 & 0xffu) | both << 8);
   }
   __syncwarp();
   // ---- the streams, one lane each
@@ -881,7 +973,7 @@ __global__ void __launch_bounds__(32) k_zstd_dec(DecParams p) {
   const uint32_t tl = z.tree_len, cs = z.cs;
   bool ok = true;
   if (z.sf == 0u) {
-    if (lane == 0) ok = read_stream(z, lit + tl, cs - tl, dst, m);
+    if (lane == 0) ok = read_stream(z, lit + tl, cs - tl, dst, m, 1u);
   } else {
     if (tl + 6u > cs) return fail();
     uint32_t sz[4];
@@ -894,7 +986,7 @@ __global__ void __launch_bounds__(32) k_zstd_dec(DecParams p) {
       uint32_t off = tl + 6u;
       for (uint32_t k = 0; k < lane; k++) off += sz[k];
       const uint32_t l0 = lane * seg, l1 = lane < 3 ? l0 + seg : m;
-      ok = read_stream(z, lit + off, sz[lane], dst + l0, l1 - l0);
+      ok = read_stream(z, lit + off, sz[lane], dst + l0, l1 - l0, 15u);
     }
   }
   if (__any_sync(0xffffffffu, !ok)) fail();
