@@ -22,10 +22,11 @@
 //   lanes    block headers validated and sized (Sec. II, PFOR blocks)
 //   then, per 256-pixel step (lane l owning the 8 consecutive pixels
 //   8l .. 8l+7 of the step), interleaved:
-//   unpack   the blocks the step needs, lane l owning the 4 consecutive
-//            values 4l..4l+3: a window of the body words they occupy,
-//            funnel-shift extraction, exception high parts via a patch
-//            buffer, inverse ZigZag (Eq. 1), into a ring of deltas
+//   unpack   the blocks the step needs, two at a time, lane l owning the 8
+//            consecutive values 8l..8l+7 of their 256 (half the instructions
+//            per value of one block and 4 values): a window of the body words
+//            they occupy, funnel-shift extraction, exception high parts via a
+//            patch buffer, inverse ZigZag (Eq. 1), into a ring of deltas
 //   scatter  compacted index of each own pixel from its mask word's; the
 //            lane's running sum of its deltas + a warp scan of the lanes'
 //            sums from the row's carry = the residuals (inverse delta); +
@@ -67,7 +68,7 @@ __device__ __forceinline__ uint32_t find_seg(const uint32_t* base, uint32_t n, u
 }  // namespace
 
 // Per-warp shared memory (byte offsets): a ring of 512 deltas (unpacked
-// ahead of the scatter), a 128-word exception patch buffer, the row's block
+// ahead of the scatter), a 256-word exception patch buffer, the row's block
 // descriptors, zero mask words (1 = zero sample), each mask word's first
 // compacted index and literal mask words.
 constexpr uint32_t kRing = 512;
@@ -80,7 +81,7 @@ __host__ __device__ inline DecWarpLayout dec_warp_layout(uint32_t W) {
   DecWarpLayout L;
   L.ring = 0;
   L.patch = L.ring + 4u * kRing;
-  L.desc = L.patch + 4u * kBlockN;
+  L.desc = L.patch + 8u * kBlockN;
   L.mw = L.desc + ((8u * ceil_div_u32(W, kBlockN) + 15u) & ~15u);
   L.wbase = L.mw + ((4u * ceil_div_u32(W, 32u) + 15u) & ~15u);
   L.lits = L.wbase + ((4u * ceil_div_u32(W, 32u) + 15u) & ~15u);
@@ -802,8 +803,8 @@ __device__ __forceinline__ void decode_item(const DecParams& p, const uint32_t k
   }
   __syncwarp();
 
-  // ---- unpack, block by block (lane l: the 4 consecutive values 4l..4l+3,
-  //      a register window of the body words they occupy, funnel-shift
+  // ---- unpack, two blocks at a time (lane l: 8 consecutive values, a
+  //      register window of the body words they occupy, funnel-shift
   //      extraction; exceptions' high parts through the patch buffer;
   //      inverse ZigZag, Eq. 1) into a ring of deltas, interleaved with the
   //      scatter by position: per 256-pixel step a warp scan of the lanes'
@@ -814,7 +815,7 @@ __device__ __forceinline__ void decode_item(const DecParams& p, const uint32_t k
     const uint32_t Pq = at.P;
     const bool no_delta = (stages & kStageNoDelta) != 0u, no_zz = (stages & kStageNoZigzag) != 0u;
     const uint32_t last_word = clen / 4u - 1u;
-    uint32_t erun = carry, blk = 0, unpacked = 0;
+    uint32_t erun = carry, unpacked = 0;
     bool xbad = false;
     for (uint32_t it = 0; it < niter && !xbad; it++) {
       const uint32_t x0 = 256u * it + 8u * lane;
@@ -825,59 +826,74 @@ __device__ __forceinline__ void decode_item(const DecParams& p, const uint32_t k
       const uint32_t nzm = ~(X >> (x0 & 31u)) & ((1u << nv) - 1u);
       uint32_t kk = nv ? wbase[x0 >> 5] + __popc(~X & ((1u << (x0 & 31u)) - 1u)) : n;
       const uint32_t kend = 8u * it + 8u < nw ? wbase[8u * it + 8u] : n;
-      while (unpacked < kend) {
-        const uint2 dsc = desc[blk];
+      while (unpacked < kend) {  // two blocks: lane l the values 8l .. 8l+7 of their 256
+        const uint32_t blk = (unpacked >> 7) + (lane >> 4), l16 = lane & 15u;
+        const uint2 dsc = blk < nb ? desc[blk] : make_uint2(0u, 0u);
         const uint32_t b = dsc.y & 0xffu, e = (dsc.y >> 8) & 0xffu, hb = (dsc.y >> 16) & 0xffu;
         const uint32_t bm = b >= 32u ? 0xffffffffu : ((1u << b) - 1u);
-        const uint32_t bit0 = 4u * lane * b, sh = bit0 & 31u;
-        const uint32_t w0 = dsc.x + (bit0 >> 5);
-        uint32_t v0 = 0, v1 = 0, v2 = 0, v3 = 0;
-        if (b) {
+        uint32_t v[8];
+        if (__all_sync(0xffffffffu, b <= 8u)) {  // 8 values in 64 bits
+          const uint32_t bit0 = 8u * l16 * b, sh = bit0 & 31u, w0 = dsc.x + (bit0 >> 5);
           const uint32_t W0 = chunk[min(w0, last_word)], W1 = chunk[min(w0 + 1u, last_word)],
                          W2 = chunk[min(w0 + 2u, last_word)];
           const uint32_t A = __funnelshift_r(W0, W1, sh), B = __funnelshift_r(W1, W2, sh);
-          if (b <= 8u) {
-            v0 = A; v1 = A >> b; v2 = A >> (2u * b); v3 = A >> (3u * b);
-          } else if (b <= 16u) {
-            const unsigned long long Y = ((unsigned long long)B << 32) | A;
-            v0 = A; v1 = __funnelshift_r(A, B, b); v2 = __funnelshift_rc(A, B, 2u * b);
-            v3 = (uint32_t)(Y >> (3u * b));
-          } else {
-            const uint32_t W3 = chunk[min(w0 + 3u, last_word)], W4 = chunk[min(w0 + 4u, last_word)];
-            const uint32_t C = __funnelshift_r(W2, W3, sh), D = __funnelshift_r(W3, W4, sh);
-            v0 = A; v1 = __funnelshift_rc(A, B, b); v2 = __funnelshift_rc(B, C, 2u * b - 32u);
-            v3 = 3u * b <= 64u ? __funnelshift_rc(B, C, 3u * b - 32u) : __funnelshift_rc(C, D, 3u * b - 64u);
+          const uint32_t C = __funnelshift_rc(A, B, 4u * b);
+          v[0] = A; v[1] = A >> b; v[2] = A >> (2u * b); v[3] = A >> (3u * b);
+          v[4] = C; v[5] = C >> b; v[6] = C >> (2u * b); v[7] = C >> (3u * b);
+        } else {  // some block is wider: 4 values in up to 128 bits, twice
+#pragma unroll
+          for (uint32_t h = 0; h < 2; h++) {
+            const uint32_t bit0 = (8u * l16 + 4u * h) * b, sh = bit0 & 31u, w0 = dsc.x + (bit0 >> 5);
+            const uint32_t W0 = chunk[min(w0, last_word)], W1 = chunk[min(w0 + 1u, last_word)],
+                           W2 = chunk[min(w0 + 2u, last_word)];
+            const uint32_t A = __funnelshift_r(W0, W1, sh), B = __funnelshift_r(W1, W2, sh);
+            uint32_t* q = v + 4u * h;
+            if (b <= 16u) {
+              const unsigned long long Y = ((unsigned long long)B << 32) | A;
+              q[0] = A; q[1] = __funnelshift_r(A, B, b); q[2] = __funnelshift_rc(A, B, 2u * b);
+              q[3] = (uint32_t)(Y >> (3u * b));
+            } else {
+              const uint32_t W3 = chunk[min(w0 + 3u, last_word)], W4 = chunk[min(w0 + 4u, last_word)];
+              const uint32_t C = __funnelshift_r(W2, W3, sh), D = __funnelshift_r(W3, W4, sh);
+              q[0] = A; q[1] = __funnelshift_rc(A, B, b); q[2] = __funnelshift_rc(B, C, 2u * b - 32u);
+              q[3] = 3u * b <= 64u ? __funnelshift_rc(B, C, 3u * b - 32u) : __funnelshift_rc(C, D, 3u * b - 64u);
+            }
           }
-          v0 &= bm; v1 &= bm; v2 &= bm; v3 &= bm;
         }
-        if (e) {  // exceptions: positions (ascending, < m), high parts of hb bits
+#pragma unroll
+        for (int i = 0; i < 8; i++) v[i] &= bm;  // (b = 0: all zero)
+        if (__any_sync(0xffffffffu, e)) {  // exceptions: positions (ascending, < m), high parts of hb bits
           const uint32_t m = dsc.y >> 24;
-          reinterpret_cast<uint4*>(patch)[lane] = make_uint4(0u, 0u, 0u, 0u);
+          uint4* pt = reinterpret_cast<uint4*>(patch) + 2u * lane;
+          pt[0] = pt[1] = make_uint4(0u, 0u, 0u, 0u);
           __syncwarp();
           const uint32_t lw = dsc.x + ((m * b + 31u) >> 5);
           const uint8_t* pos = reinterpret_cast<const uint8_t*>(chunk + lw);
           const uint32_t hw = lw + ((e + 3u) >> 2);
           const uint32_t hmask = hb >= 32u ? 0xffffffffu : ((1u << hb) - 1u);
-          for (uint32_t jx = lane; jx < e; jx += 32) {
+          for (uint32_t jx = l16; jx < e; jx += 16) {
             const uint32_t ps = pos[jx];
             if (ps >= m || (jx > 0 && ps <= pos[jx - 1])) {
               xbad = true;
             } else {
               const uint32_t bit = jx * hb, wi = hw + (bit >> 5);
               const uint32_t lo = chunk[min(wi, last_word)], hi = chunk[min(wi + 1u, last_word)];
-              patch[ps] = (__funnelshift_r(lo, hi, bit & 31u) & hmask) << b;
+              patch[128u * (lane >> 4) + ps] = (__funnelshift_r(lo, hi, bit & 31u) & hmask) << b;
             }
           }
           __syncwarp();
-          const uint4 pt = reinterpret_cast<const uint4*>(patch)[lane];
-          v0 |= pt.x; v1 |= pt.y; v2 |= pt.z; v3 |= pt.w;
+          const uint4 p0 = pt[0], p1 = pt[1];
+          v[0] |= p0.x; v[1] |= p0.y; v[2] |= p0.z; v[3] |= p0.w;
+          v[4] |= p1.x; v[5] |= p1.y; v[6] |= p1.z; v[7] |= p1.w;
         }
         if (!no_zz) {
-          v0 = unzigzag(v0); v1 = unzigzag(v1); v2 = unzigzag(v2); v3 = unzigzag(v3);
+#pragma unroll
+          for (int i = 0; i < 8; i++) v[i] = unzigzag(v[i]);
         }
-        reinterpret_cast<uint4*>(ring)[((128u * blk + 4u * lane) & (kRing - 1u)) >> 2] = make_uint4(v0, v1, v2, v3);
-        unpacked += min(kBlockN, n - 128u * blk);
-        blk++;
+        uint4* rp = reinterpret_cast<uint4*>(ring) + (((unpacked + 8u * lane) & (kRing - 1u)) >> 2);
+        rp[0] = make_uint4(v[0], v[1], v[2], v[3]);
+        rp[1] = make_uint4(v[4], v[5], v[6], v[7]);
+        unpacked += 2u * kBlockN;
       }
       xbad = __any_sync(0xffffffffu, xbad);
       __syncwarp();

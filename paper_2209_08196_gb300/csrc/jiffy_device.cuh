@@ -73,13 +73,13 @@ __device__ __forceinline__ void store_sample(uint8_t* row, uint32_t s, uint32_t 
   else row[x] = (uint8_t)v;
 }
 
-__device__ __forceinline__ uint32_t warp_incl_scan_fwd(uint32_t v) {
-  const uint32_t lane = threadIdx.x & 31u;
+// Inclusive prefix sum over the warp; the shuffle itself says which lanes
+// have a source (no lane compares).
+__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= (uint32_t)o) v += t;
-  }
+  for (int o = 1; o < 32; o <<= 1)
+    asm("{\n\t.reg .pred p;\n\t.reg .u32 t;\n\tshfl.sync.up.b32 t|p, %0, %1, 0, 0xffffffff;\n\t@p add.u32 %0, %0, t;\n\t}"
+        : "+r"(v) : "r"(o));
   return v;
 }
 
@@ -233,7 +233,7 @@ __device__ __forceinline__ void store8s(uint8_t* row, uint32_t x0, uint32_t nval
 }
 
 __device__ __forceinline__ uint32_t warp_excl_scan(uint32_t v, uint32_t& total) {
-  const uint32_t incl = warp_incl_scan_fwd(v);
+  const uint32_t incl = warp_incl_scan(v);
   total = __shfl_sync(0xffffffffu, incl, 31);
   return incl - v;
 }
@@ -288,16 +288,6 @@ __device__ __forceinline__ uint32_t block_body_bytes(uint32_t n, uint32_t b, uin
   uint32_t bytes = 4u * ((n * b + 31u) >> 5);
   if (e) bytes += 4u * ((e + 3u) >> 2) + 4u * ((e * (wmax - b) + 31u) >> 5);
   return bytes;
-}
-
-__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
-  const uint32_t lane = lane_id();
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= (uint32_t)o) v += t;
-  }
-  return v;
 }
 
 __device__ __forceinline__ uint32_t warp_sum(uint32_t v) { return __reduce_add_sync(0xffffffffu, v); }
