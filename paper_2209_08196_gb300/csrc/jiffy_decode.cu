@@ -26,13 +26,13 @@
 //            consecutive values 8l..8l+7 of their 256 (half the instructions
 //            per value of one block and 4 values): a window of the body words
 //            they occupy, funnel-shift extraction, exception high parts via a
-//            patch buffer, inverse ZigZag (Eq. 1), into a ring of deltas
-//   scatter  compacted index of each own pixel from its mask word's; the
-//            lane's running sum of its deltas + a warp scan of the lanes'
-//            sums from the row's carry = the residuals (inverse delta); +
-//            previous pixel for P; x precision (Sec. III-A); vector stores
+//            patch buffer, inverse ZigZag (Eq. 1); running sums and a warp
+//            scan from the row's carry (inverse delta, on the kept samples
+//            alone), into a ring of residuals
+//   scatter  compacted index of each own pixel from its mask word's; x
+//            precision (Sec. III-A); + previous pixel for P; vector stores
 // The row chunk is read through L1 (bulk-prefetched into L2 at the start of
-// the row); deltas pass through a small ring buffer in shared memory.
+// the row); residuals pass through a small ring buffer in shared memory.
 #include <algorithm>
 
 #include "jiffy_device.cuh"
@@ -67,8 +67,8 @@ __device__ __forceinline__ uint32_t find_seg(const uint32_t* base, uint32_t n, u
 
 }  // namespace
 
-// Per-warp shared memory (byte offsets): a ring of 512 deltas (unpacked
-// ahead of the scatter), a 256-word exception patch buffer, the row's block
+// Per-warp shared memory (byte offsets): a ring of 512 residuals (unpacked
+// ahead of the scatter; the first 8 again behind the last), a 256-word exception patch buffer, the row's block
 // descriptors, zero mask words (1 = zero sample), each mask word's first
 // compacted index and literal mask words.
 constexpr uint32_t kRing = 512;
@@ -80,7 +80,7 @@ struct DecWarpLayout {
 __host__ __device__ inline DecWarpLayout dec_warp_layout(uint32_t W) {
   DecWarpLayout L;
   L.ring = 0;
-  L.patch = L.ring + 4u * kRing;
+  L.patch = L.ring + 4u * (kRing + 8u);
   L.desc = L.patch + 8u * kBlockN;
   L.mw = L.desc + ((8u * ceil_div_u32(W, kBlockN) + 15u) & ~15u);
   L.wbase = L.mw + ((4u * ceil_div_u32(W, 32u) + 15u) & ~15u);
@@ -806,10 +806,9 @@ __device__ __forceinline__ void decode_item(const DecParams& p, const uint32_t k
   // ---- unpack, two blocks at a time (lane l: 8 consecutive values, a
   //      register window of the body words they occupy, funnel-shift
   //      extraction; exceptions' high parts through the patch buffer;
-  //      inverse ZigZag, Eq. 1) into a ring of deltas, interleaved with the
-  //      scatter by position: per 256-pixel step a warp scan of the lanes'
-  //      delta sums from the running residual is the inverse delta; + the
-  //      previous pixel for P, x precision (Sec. III-A)
+  //      inverse ZigZag, Eq. 1; inverse delta from the running residual) into
+  //      a ring of residuals, interleaved with the scatter by position: x
+  //      precision (Sec. III-A), + the previous pixel for P
   if (chained && !summed && !bad) wait_row(2u);
   if (!bad) {
     const uint32_t Pq = at.P;
@@ -824,7 +823,7 @@ __device__ __forceinline__ void decode_item(const DecParams& p, const uint32_t k
       // compacted index of the first; the step ends at the next word group
       const uint32_t X = nv ? mw[x0 >> 5] : 0xffffffffu;
       const uint32_t nzm = ~(X >> (x0 & 31u)) & ((1u << nv) - 1u);
-      uint32_t kk = nv ? wbase[x0 >> 5] + __popc(~X & ((1u << (x0 & 31u)) - 1u)) : n;
+      const uint32_t kk = nv ? wbase[x0 >> 5] + __popc(~X & ((1u << (x0 & 31u)) - 1u)) : n;
       const uint32_t kend = 8u * it + 8u < nw ? wbase[8u * it + 8u] : n;
       while (unpacked < kend) {  // two blocks: lane l the values 8l .. 8l+7 of their 256
         const uint32_t blk = (unpacked >> 7) + (lane >> 4), l16 = lane & 15u;
@@ -890,9 +889,24 @@ __device__ __forceinline__ void decode_item(const DecParams& p, const uint32_t k
 #pragma unroll
           for (int i = 0; i < 8; i++) v[i] = unzigzag(v[i]);
         }
-        uint4* rp = reinterpret_cast<uint4*>(ring) + (((unpacked + 8u * lane) & (kRing - 1u)) >> 2);
+        if (!no_delta) {  // deltas to residuals: running sums from the last one (values past n follow it)
+          uint32_t sum = v[0];
+#pragma unroll
+          for (int i = 1; i < 8; i++) sum += v[i];
+          uint32_t tot;
+          v[0] += erun + warp_excl_scan(sum, tot);
+          erun += tot;
+#pragma unroll
+          for (int i = 1; i < 8; i++) v[i] += v[i - 1];
+        }
+        const uint32_t at = (unpacked + 8u * lane) & (kRing - 1u);
+        uint4* rp = reinterpret_cast<uint4*>(ring) + (at >> 2);
         rp[0] = make_uint4(v[0], v[1], v[2], v[3]);
         rp[1] = make_uint4(v[4], v[5], v[6], v[7]);
+        if (at == 0u) {  // again behind the end, for the 8 pixels of a lane that run past it
+          rp[kRing / 4u] = rp[0];
+          rp[kRing / 4u + 1u] = rp[1];
+        }
         unpacked += 2u * kBlockN;
       }
       xbad = __any_sync(0xffffffffu, xbad);
@@ -900,33 +914,14 @@ __device__ __forceinline__ void decode_item(const DecParams& p, const uint32_t k
       if (xbad) break;
       uint32_t pv[8] = {0, 0, 0, 0, 0, 0, 0, 0};
       if (prow && nv) load8<true>(prow, S, x0, nv, vec_prev, pv);
-      // residuals: running sum of the deltas from the step's start (without
-      // the delta stage the values are the residuals)
-      uint32_t d[8], ebase = 0;
-      if (!no_delta) {
-        uint32_t lsum = 0;
-#pragma unroll
-        for (int i = 0; i < 8; i++) {
-          const bool nzb = (nzm >> i) & 1u;
-          d[i] = nzb ? ring[kk & (kRing - 1u)] : 0u;
-          kk += nzb ? 1u : 0u;
-          lsum += d[i];
-          d[i] = lsum;
-        }
-        uint32_t stot;
-        ebase = erun + warp_excl_scan(lsum, stot);
-        erun += stot;
-      } else {
-#pragma unroll
-        for (int i = 0; i < 8; i++) {
-          const bool nzb = (nzm >> i) & 1u;
-          d[i] = nzb ? ring[kk & (kRing - 1u)] : 0u;
-          kk += nzb ? 1u : 0u;
-        }
-      }
       uint32_t out[8];
+      const uint32_t* res = ring + (kk & (kRing - 1u));
 #pragma unroll
-      for (int i = 0; i < 8; i++) out[i] = ((nzm >> i) & 1u) ? (ebase + d[i]) * Pq + pv[i] : 0u;
+      for (int i = 0; i < 8; i++) {
+        const bool kept = (nzm >> i) & 1u;
+        out[i] = kept ? *res * Pq + pv[i] : 0u;
+        res += kept ? 1 : 0;
+      }
       if (nv) {
         store8(orow, S, x0, nv, vec_out, out);
         if (srow) store8(srow, S, x0, nv, vec_out, out);
@@ -944,8 +939,9 @@ __device__ __forceinline__ void decode_item(const DecParams& p, const uint32_t k
   }
 }
 
+// (at most 64 registers: 32 warps per SM)
 template <int WPC, bool STAGED, bool LOCAL>
-__global__ void __launch_bounds__(WPC * 32) k_decode(DecParams p) {
+__global__ void __launch_bounds__(WPC * 32, 32 / WPC) k_decode(DecParams p) {
   extern __shared__ __align__(16) uint32_t smem[];
   const uint32_t lane = lane_id();
   const DecWarpLayout lay = dec_warp_layout(p.max_W);
