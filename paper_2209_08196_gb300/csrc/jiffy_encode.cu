@@ -124,6 +124,9 @@ __device__ __forceinline__ uint32_t zigzag_small(uint32_t d) {
 
 // (precisions without a 32-bit multiplier, out of line: 64-bit products)
 __device__ __noinline__ uint32_t quant_wide(uint32_t v, const AttrDev& at) { return quant<2>(v, at); }
+__device__ __forceinline__ uint32_t quant_any(uint32_t v, const AttrDev& at) {
+  return at.qkind == 0 ? v : at.qkind == 1 ? quant<1>(v, at) : quant_wide(v, at);
+}
 __device__ __forceinline__ void quant8_wide(uint32_t (&v)[8], const AttrDev& at) {
 #pragma unroll
   for (int i = 0; i < 8; i++) v[i] = quant_wide(v[i], at);
@@ -257,13 +260,12 @@ __device__ __noinline__ bool row_last(const uint8_t* cur, const uint8_t* prv, co
   return false;
 }
 
-// Values n .. (end of the last 1024-value step) repeat `last` (the last
+// Values n .. (end of their 32-value segment) repeat `last` (the last
 // residual, or 0 without the delta stage), so that their deltas are 0 and
-// they count as zero-width values.
+// they count as zero-width values. (Segments past n are not looked at.)
 __device__ __forceinline__ void fill_tail(uint32_t* zb, uint32_t n, uint32_t last) {
-  const uint32_t end = (n + kStepVal - 1) / kStepVal * kStepVal;
-#pragma unroll 1
-  for (uint32_t k = n + lane_id(); k < end; k += 32u) zb[zaddr(k)] = last;
+  const uint32_t k = n + lane_id();
+  if (k < ((n + 31u) & ~31u)) zb[zaddr(k)] = last;
   __syncwarp();
 }
 
@@ -391,15 +393,20 @@ __device__ __forceinline__ uint32_t block_width(const uint32_t (&A)[6], uint32_t
   return key;
 }
 
-// Delta, ZigZag and column counts of a step: the lanes' segments zs, the first
-// of which continues pred_step (updated to the step's last residual). fast:
+// Delta, ZigZag and column counts of a step: the lanes' segments zs (active:
+// with values in them; the others count nothing), the first of which continues
+// pred_step (updated to the step's last residual). fast:
 // every delta is below 2^30 in magnitude (zigzag_small). st: stage switches.
 template <bool STAGED>
-__device__ __forceinline__ void step_planes(uint32_t* zs, uint32_t& pred_step, bool fast, uint32_t st, uint32_t (&P)[6]) {
-  const uint32_t last = zs[31];
+__device__ __forceinline__ void step_planes(uint32_t* zs, bool active, uint32_t& pred_step, bool fast, uint32_t st,
+                                            uint32_t (&P)[6]) {
+  const uint32_t last = active ? zs[31] : 0u;
   uint32_t pred = __shfl_up_sync(kFull, last, 1);
   if (lane_id() == 0) pred = pred_step;
   pred_step = __shfl_sync(kFull, last, 31);
+#pragma unroll
+  for (int k = 0; k < 6; k++) P[k] = 0u;
+  if (!active) return;
   if (fast && !(STAGED && (st & (kStageNoDelta | kStageNoZigzag)))) {
     seg_planes<true>(zs, pred, P);
   } else {
@@ -419,7 +426,8 @@ __device__ __forceinline__ uint32_t price_row(uint32_t* zb, uint32_t n, uint32_t
     const uint32_t seg = (s0 >> 5) + lane;
     uint32_t* zs = zb + kSegWords * seg;
     uint32_t P[6];
-    step_planes<true>(zs, pred_step, fast, st, P);
+    step_planes<true>(zs, 32u * seg < n, pred_step, fast, st, P);
+    __syncwarp();
     const uint32_t g = seg >> 2;
     const uint32_t m = n > 128u * g ? min(128u, n - 128u * g) : 0u;
     uint32_t wmax;
@@ -564,7 +572,9 @@ __device__ __forceinline__ uint32_t code_step(uint32_t* zb, uint32_t s0, uint32_
   const uint32_t seg = (s0 >> 5) + lane;
   uint32_t* zs = zb + kSegWords * seg;
   uint32_t P[6];
-  step_planes<STAGED>(zs, pred_step, fast, st, P);
+  const bool active = 32u * seg < n;
+  step_planes<STAGED>(zs, active, pred_step, fast, st, P);
+  __syncwarp();
   const uint32_t g = seg >> 2;
   const uint32_t m = n > 128u * g ? min(128u, n - 128u * g) : 0u;
   uint32_t wmax;
@@ -582,7 +592,7 @@ __device__ __forceinline__ uint32_t code_step(uint32_t* zb, uint32_t s0, uint32_
   uint32_t* wp = reinterpret_cast<uint32_t*>(blk) + j * b;
   if (__any_sync(kFull, e != 0u)) {
     const uint32_t xm = pack_low<true>(zs, b, lim, wp);
-    pack_exceptions(xm, zs, j, b, e, hb, blk, low_words);
+    pack_exceptions(active ? xm : 0u, zs, j, b, e, hb, blk, low_words);
   } else {
     pack_low<false>(zs, b, lim, wp);
   }
@@ -685,24 +695,15 @@ struct EncWarp {
   uint8_t* mb;
 };
 
-// The last kept sample among the 8 (nv valid) in v / pv, across the warp:
-// its residual (P: q - q', I: q). Returns false if there is none.
-__device__ __forceinline__ bool tail_residual(uint32_t (&v)[8], uint32_t (&pv)[8], uint32_t nv, bool pm, bool all,
-                                              const AttrDev& at, uint32_t& e_last) {
-  quant8(v, at);
-  if (pm) quant8(pv, at);
-  bool has = false;
-  uint32_t last = 0;
-#pragma unroll
-  for (int i = 0; i < 8; i++) {
-    if ((uint32_t)i < nv && (v[i] != 0u || all)) {
-      has = true;
-      last = pm ? v[i] - pv[i] : v[i];
-    }
-  }
-  const uint32_t hm = __ballot_sync(kFull, has);
+// The residual (P: q - q', I: q) of the last kept sample among the 32 samples
+// v (P: pv) of a warp, `in` the lanes that hold one. Returns false if there is
+// none.
+__device__ __forceinline__ bool last_residual(uint32_t v, uint32_t pv, bool in, bool pm, bool all, const AttrDev& at,
+                                              uint32_t& e_last) {
+  const uint32_t q = quant_any(v, at), e = pm ? q - quant_any(pv, at) : q;
+  const uint32_t hm = __ballot_sync(kFull, in && (q != 0u || all));
   if (!hm) return false;
-  e_last = __shfl_sync(kFull, last, 31u - __clz(hm));
+  e_last = __shfl_sync(kFull, e, 31u - __clz(hm));
   return true;
 }
 
@@ -731,15 +732,13 @@ __device__ __forceinline__ void encode_item(const EncParams& p, const uint32_t k
     prefetch_l2(cur, rowb);
     if (prv) prefetch_l2(prv, rowb);
   }
-  // the previous row's last 256-pixel step, loaded now and read after pass A:
-  // its last kept residual is this row's delta carry (Sec. III-C)
-  const uint32_t nsteps = ceil_div_u32(W, kStepPx);
-  const uint32_t tx0 = kStepPx * (nsteps - 1u) + 8u * lane;
-  const uint32_t tnv = tx0 < W ? min(8u, W - tx0) : 0u;
-  uint32_t tv[8], tpv[8];
-  if (r > 0) {
-    load8<false>(cur - rowb, at.s, tx0, tnv, vec_ok(cur - rowb, at.s), tv);
-    if (prv) load8<false>(prv - rowb, at.s, tx0, tnv, vec_ok(prv - rowb, at.s), tpv);
+  // the previous row's last 32 pixels, loaded now and read after pass A: its
+  // last kept residual is this row's delta carry (Sec. III-C)
+  const int tx = (int)W - 32 + (int)lane;
+  uint32_t tv = 0, tpv = 0;
+  if (r > 0 && tx >= 0) {
+    tv = load_sample(cur - rowb, at.s, (uint32_t)tx);
+    if (prv) tpv = load_sample(prv - rowb, at.s, (uint32_t)tx);
   }
 
   // ---- pass A
@@ -770,7 +769,15 @@ __device__ __forceinline__ void encode_item(const EncParams& p, const uint32_t k
   uint32_t carry = 0;
   bool known = r == 0;  // e[-1] = 0 at the start of the attribute-scan
   if (r > 0) {
-    known = tail_residual(tv, tpv, tnv, prv != nullptr, kz == 0u, at, carry);
+    known = last_residual(tv, tpv, tx >= 0, prv != nullptr, kz == 0u, at, carry);
+#pragma unroll 1
+    for (int k = 1; !known && k < 8; k++) {  // 7 times 32 pixels more
+      const int x = tx - 32 * k;
+      const bool in = x >= 0;
+      const uint32_t v = in ? load_sample(cur - rowb, at.s, (uint32_t)x) : 0u;
+      const uint32_t pv = in && prv ? load_sample(prv - rowb, at.s, (uint32_t)x) : 0u;
+      known = last_residual(v, pv, in, prv != nullptr, kz == 0u, at, carry);
+    }
   }
   if (!known) {  // the previous rows' "last residual" words decide
     const bool ok = lookback_last(p.st_carry, k, sec_start, carry);
