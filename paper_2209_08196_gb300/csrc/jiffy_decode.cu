@@ -130,15 +130,15 @@ __device__ __forceinline__ DecSec find_section(const DecSeg& sg, uint32_t t, uin
       }
     }
     s.data_len = mine - 8u * H - s.zpart;
-    if (stream_header && t == 0 && a == 0 && sg.check_shdr && !bad) {  // stream header: shape, dtypes, precisions
-      if (ld_in_u32(sg.in, 0) != 0x3159464Au || ld_in_u32(sg.in, 4) != (1u | (A << 16)) ||
-          ld_in_u32(sg.in, 8) != H || ld_in_u32(sg.in, 12) != sg.W)
-        bad = true;
-      for (uint32_t aa = 0; aa < A && !bad; aa++) {
-        if (ld_in_u32(sg.in, 16 + 8ull * aa) != attr_header_word(sg.attrs[aa].s, sg.stages) ||
-            ld_in_u32(sg.in, 20 + 8ull * aa) != sg.attrs[aa].P)
-          bad = true;
-      }
+    if (stream_header && t == 0 && a == 0 && sg.check_shdr && !bad) {
+      // stream header: shape, dtypes, precisions (compared without a branch
+      // in between, so that the words are read together)
+      uint32_t diff = (ld_in_u32(sg.in, 0) ^ 0x3159464Au) | (ld_in_u32(sg.in, 4) ^ (1u | (A << 16))) |
+                      (ld_in_u32(sg.in, 8) ^ H) | (ld_in_u32(sg.in, 12) ^ sg.W);
+      for (uint32_t aa = 0; aa < A; aa++)
+        diff |= (ld_in_u32(sg.in, 16 + 8ull * aa) ^ attr_header_word(sg.attrs[aa].s, sg.stages)) |
+                (ld_in_u32(sg.in, 20 + 8ull * aa) ^ sg.attrs[aa].P);
+      bad = diff != 0u;
     }
   }
   if (bad) s = DecSec{};
@@ -362,7 +362,8 @@ __device__ __forceinline__ void undo_masks(const DecParams& p, const DecSeg& sg,
   for (uint32_t T0 = 0; T0 < T; T0 += kMaskThreads) {
     const uint32_t t = T0 + tid;
     const uint32_t pm = frame_mode(p, sg, a, t);
-    const bool need = t < T && (pm || frame_mode(p, sg, a, t + 1u));
+    const bool goes_on = frame_mode(p, sg, a, t + 1u) != 0u;
+    const bool need = t < T && (pm || goes_on);
     MaskWords mw{nullptr, 0u, ncls, nullptr, sg.zm_rb};
     if (need && zmask) {
       mw.zrow = p.zdec + sg.zm_base + (size_t)(t * sg.A + a) * sg.zm_stride + (size_t)r * sg.zm_rb;
@@ -400,7 +401,8 @@ __device__ __forceinline__ void undo_masks(const DecParams& p, const DecSeg& sg,
     };
     const uint32_t last_valid = valid_word_bits(W, nw, nw - 1u);
     if (!ONE && T - T0 > 32u) {  // the warps' last masks, as if nothing came before them; then each warp's carry
-      if (needs) {
+      // (where the next warp's first frame continues a run)
+      if (__shfl_sync(0xffffffffu, (uint32_t)goes_on, 31)) {
         MaskWords m = mw;
         const uint32_t none[4] = {0, 0, 0, 0};
         for (uint32_t j = j0; j < j1; j += 4u) {
