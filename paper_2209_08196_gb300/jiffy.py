@@ -9,6 +9,7 @@ fallback: without the built library every call raises.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 
@@ -125,7 +126,7 @@ def _lib() -> ctypes.CDLL:
         L.jiffy_decode_batch_async.argtypes = L.jiffy_decode_batch.argtypes
         L.jiffy_batch_wait.restype = ctypes.c_int
         L.jiffy_batch_wait.argtypes = [vp]
-        # the same batched entry points over plain addresses (arguments marshalled as numpy arrays)
+        # the same batched entry points over plain addresses (arguments marshalled as arrays)
         for name, n_ptr in (("jiffy_encode_batch", 9), ("jiffy_decode_batch", 8)):
             for f in (name, name + "_async"):
                 _BATCH_ADDR[f] = ctypes.CFUNCTYPE(ctypes.c_int, vp, u32, *([vp] * n_ptr))((f, L))
@@ -512,22 +513,23 @@ def jiffy_stream_device_bytes(h: Handle) -> int:
 
 
 def _batch_tables(handles, planes, what: str):
-    """(scans per stream, plane pointer tables of all streams in one uint64
-    array, where each stream's table starts). Planes are given and checked per
-    stream as for the sequence calls (_seq_ptrs); the pointers of all streams
-    are computed at once (64 streams: a table of their own each took some 5 us
-    a stream)."""
-    counts, bases, steps, per_scan, scans = [], [], [], [], []
+    """(scans per stream, plane pointer tables of all streams in one array of
+    64-bit words, where each stream's table starts). Planes are given and
+    checked per stream as for the sequence calls (_seq_ptrs). Many pointers
+    are computed as numpy arrays (64 streams, 800 pointers: 25 us instead of
+    50), a few as a list."""
+    counts, bases, steps, per_scan, scans, starts = [], [], [], [], [], []
+    total = 0
     for h, pl in zip(handles, planes):
         p0 = pl[0]
         attrs = h.attrs
         if isinstance(p0, torch.Tensor) and len(pl) == len(attrs) and p0.dim() == 3:
             T, HW = p0.shape[0], h.H * h.W
-            for p, (s, _) in zip(pl, attrs):
+            for a, (p, (s, _)) in enumerate(zip(pl, attrs)):
                 sh = p.shape
                 if sh[0] != T or not p.is_cuda or p.element_size() != s or not p.is_contiguous() or sh[1] * sh[2] != HW:
                     raise ValueError("%s %d: expected a contiguous CUDA tensor of %d x %d x %d %d-byte samples, got %s %s"
-                                     % (what, len(bases) - sum(per_scan), T, h.H, h.W, s, tuple(sh), p.dtype))
+                                     % (what, a, T, h.H, h.W, s, tuple(sh), p.dtype))
                 bases.append(p.data_ptr())
                 steps.append(HW * s)
             per_scan.append(len(pl))
@@ -541,65 +543,82 @@ def _batch_tables(handles, planes, what: str):
             per_scan.append(len(flat))
             scans.append(1)
         counts.append(T)
+        starts.append(total)
+        total += per_scan[-1] * scans[-1]
+    if total <= 256:
+        ptrs, b0 = [], 0
+        for A, T in zip(per_scan, scans):
+            pairs = list(zip(bases[b0:b0 + A], steps[b0:b0 + A]))
+            ptrs.extend([base + t * step for t in range(T) for base, step in pairs])
+            b0 += A
+        return counts, array.array("Q", ptrs), starts
     A, T = np.array(per_scan, dtype=np.int64), np.array(scans, dtype=np.int64)
     n = A * T  # pointers of each stream, scan-major
-    ends = np.cumsum(n)
-    starts = ends - n
-    k = np.arange(int(ends[-1]) if len(n) else 0, dtype=np.int64) - np.repeat(starts, n)
+    k = np.arange(total, dtype=np.int64) - np.repeat(np.array(starts, dtype=np.int64), n)
     t, a = np.divmod(k, np.repeat(A, n))
     at = np.repeat(np.cumsum(A) - A, n) + a
     table = np.array(bases, dtype=np.uint64)[at] + (np.array(steps, dtype=np.int64)[at] * t).astype(np.uint64)
-    return counts, table, starts
+    return counts, array.array("Q", table.tobytes()), starts
 
 
 def _offset_starts(counts):
-    n = np.array(counts, dtype=np.int64) + 1
-    return np.cumsum(n) - n
-
-
-def _per_stream(values, n: int, dtype=np.uint64):
-    """One value per stream; missing ones are 0 (the C ABI refuses them)."""
-    if len(values) > n:
-        raise IndexError("more arguments than streams")
-    out = np.zeros(n, dtype=dtype)
-    out[:len(values)] = values
+    out, at = [], 0
+    for c in counts:
+        out.append(at)
+        at += c + 1
     return out
 
 
-def _handle_ptrs(handles):
-    return np.array([h.ptr or 0 for h in handles], dtype=np.uint64)
+def _padded(values, n: int):
+    """One value per stream; missing ones are 0 (the C ABI refuses them)."""
+    if len(values) > n:
+        raise IndexError("more arguments than streams")
+    return values + [0] * (n - len(values))
+
+
+def _at(a, items) -> list:
+    """Addresses of elements of an array of 64-bit words."""
+    base = a.buffer_info()[0]
+    return [base + 8 * i for i in items]
 
 
 class _EncCall:
-    """Marshalled arguments of one batched encode (kept alive until it ends)."""
+    """Marshalled arguments of one batched encode (kept alive until it ends):
+    words holds n words each of stream handles, plane tables, outputs,
+    capacities, offset arrays and (results) stream bytes."""
 
     def __init__(self, handles, planes, outs):
-        n = len(handles)
+        n = self.n = len(handles)
         counts, self.table, starts = _batch_tables(handles, planes, "plane")
-        self.n = n
-        self.streams = _handle_ptrs(handles)
-        self.n_scans = _per_stream(counts, n, np.uint32)
-        self.planes = _per_stream(self.table.ctypes.data + 8 * starts, n)
-        self.outs = _per_stream([o.data_ptr() for o in outs], n)
-        self.caps = _per_stream([o.numel() * o.element_size() for o in outs], n)
-        self.ostarts = _offset_starts(counts)
-        self.offs = np.zeros(sum(counts) + n, dtype=np.uint64)
-        self.offs_pp = _per_stream(self.offs.ctypes.data + 8 * self.ostarts, n)
-        self.lens = np.zeros(n, dtype=np.uint64)
-        self.sts = np.zeros(n, dtype=np.int32)
+        self.counts, self.ostarts = counts, _offset_starts(counts)
+        self.offs = array.array("Q", bytes(8 * (sum(counts) + n)))
+        self.n_scans = array.array("I", _padded(counts, n))
+        self.sts = array.array("i", bytes(4 * n))
+        self.words = array.array("Q", [h.ptr or 0 for h in handles] + _padded(_at(self.table, starts), n)
+                                 + _padded([o.data_ptr() for o in outs], n)
+                                 + _padded([o.numel() * o.element_size() for o in outs], n)
+                                 + _padded(_at(self.offs, self.ostarts), n) + [0] * n)
+
+    @property
+    def lens(self):
+        return self.words[5 * self.n:]
 
     def args(self, b, stream):
-        return (b.ptr, self.n, *(x.ctypes.data for x in (self.streams, self.n_scans, self.planes, self.outs, self.caps,
-                                                         self.offs_pp, self.lens, self.sts)), _stream_ptr(stream))
+        w, step = self.words.buffer_info()[0], 8 * self.n
+        return (b.ptr, self.n, w, self.n_scans.buffer_info()[0], w + step, w + 2 * step, w + 3 * step, w + 4 * step,
+                w + 5 * step, self.sts.buffer_info()[0], _stream_ptr(stream))
 
     def result(self):
         offs, lens = self.offs.tolist(), self.lens.tolist()
-        return [(lens[i], offs[o:o + int(c) + 1]) for i, (o, c) in enumerate(zip(self.ostarts.tolist(), self.n_scans))]
+        return [(lens[i], offs[o:o + c + 1]) for i, (o, c) in enumerate(zip(self.ostarts, self.counts))]
 
 
 class _DecCall:
+    """As _EncCall: words holds stream handles, inputs, lengths, offset arrays
+    and plane tables."""
+
     def __init__(self, handles, bufs, lengths, offsets, planes_out):
-        n = len(handles)
+        n = self.n = len(handles)
         counts, self.table, starts = _batch_tables(handles, planes_out, "output plane")
         flat, given = [], []
         for T, o in zip(counts, offsets):
@@ -607,19 +626,18 @@ class _DecCall:
                 raise ValueError("need T + 1 frame offsets")
             flat.extend([int(v) for v in o])
             given.append(T)
-        self.n = n
-        self.streams = _handle_ptrs(handles)
-        self.n_frames = _per_stream(counts, n, np.uint32)
-        self.ins = _per_stream([x.data_ptr() for x in bufs], n)
-        self.lens = _per_stream([int(x) for x in lengths], n)
-        self.offs = np.array(flat, dtype=np.uint64)
-        self.offs_pp = _per_stream(self.offs.ctypes.data + 8 * _offset_starts(given), n)
-        self.planes = _per_stream(self.table.ctypes.data + 8 * starts, n)
-        self.sts = np.zeros(n, dtype=np.int32)
+        self.offs = array.array("Q", flat)
+        self.n_frames = array.array("I", _padded(counts, n))
+        self.sts = array.array("i", bytes(4 * n))
+        self.words = array.array("Q", [h.ptr or 0 for h in handles] + _padded([x.data_ptr() for x in bufs], n)
+                                 + _padded([int(x) for x in lengths], n)
+                                 + _padded(_at(self.offs, _offset_starts(given)), n)
+                                 + _padded(_at(self.table, starts), n))
 
     def args(self, b, stream):
-        return (b.ptr, self.n, *(x.ctypes.data for x in (self.streams, self.n_frames, self.ins, self.lens, self.offs_pp,
-                                                         self.planes, self.sts)), _stream_ptr(stream))
+        w, step = self.words.buffer_info()[0], 8 * self.n
+        return (b.ptr, self.n, w, self.n_frames.buffer_info()[0], w + step, w + 2 * step, w + 3 * step, w + 4 * step,
+                self.sts.buffer_info()[0], _stream_ptr(stream))
 
 
 def jiffy_encode_batch(b: Batch, handles, planes, outs, stream=None):
