@@ -309,9 +309,10 @@ jiffy_status jiffy_stream_set_profiling(jiffy_stream* s, int enable);
 
 /* Device milliseconds of each kernel launched by the stream's last
  * successful call, in launch order (encode: trial, rows, placement; decode:
- * rows); after jiffy_stream_wait, the averages over the enqueue-only calls
- * since the previous wait. Writes min(n, count) values to ms (host) and
- * returns the count (0 if profiling is off or no call completed). */
+ * the rows with the kernels around them); after jiffy_stream_wait, the
+ * averages over the enqueue-only calls since the previous wait. Writes
+ * min(n, count) values to ms (host) and returns the count (0 if profiling is
+ * off or no call completed). */
 uint32_t jiffy_stream_kernel_times(const jiffy_stream* s, float* ms, uint32_t n);
 
 /* Allocation-free decode of one frame, for callers that may not allocate
@@ -368,10 +369,11 @@ jiffy_status jiffy_stream_copy_state(jiffy_stream* dst, const jiffy_stream* src,
 /* Failure-detection test hook (the failure is made on the host; nothing
  * faults): in the stream's next call, row item `row_item` -- numbered
  * (a * n_scans + t) * H + r over the call's scans t, attributes a and rows r
- * -- does not publish its status: a decoder row its completion (waited on
- * before the row's P frames are added up), an encoder row its last residual (waited
- * on by the next row when that row's previous-row tail holds no nonzero
- * sample). The wait gives up after the bounded device wait (2 s); the call then returns JIFFY_ERR_TIMEOUT, the stream's
+ * -- does not publish its status: a decoder row its completion (waited on by
+ * the same row of the next frame when that is a P row), an encoder row its
+ * last residual (waited on by the next row when that row's previous-row tail
+ * holds no nonzero sample). A row that waits on it gives up after the bounded
+ * device wait (2 s); the call then returns JIFFY_ERR_TIMEOUT, the stream's
  * state stays unchanged and the device stays usable. Applies to one call.
  * Errors: INVALID_ARG. */
 jiffy_status jiffy_stream_test_withhold_row(jiffy_stream* s, uint32_t row_item);

@@ -181,57 +181,6 @@ __device__ __forceinline__ void store8(uint8_t* row, uint32_t s, uint32_t x0, ui
   store8_slow(row, s, x0, nvalid, tmp);
 }
 
-// Compile-time sample width variants (S = 1, 2 or 4 bytes).
-template <uint32_t S, bool CG>
-__device__ __forceinline__ void load8s(const uint8_t* row, uint32_t x0, uint32_t nvalid, bool vec, uint32_t (&v)[8]) {
-  if (vec && nvalid == 8) {
-    if constexpr (S == 4) {
-      const uint4* q = reinterpret_cast<const uint4*>(row + 4ull * x0);
-      const uint4 a = CG ? __ldcg(q) : q[0];
-      const uint4 b = CG ? __ldcg(q + 1) : q[1];
-      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-    } else if constexpr (S == 2) {
-      const uint4* q = reinterpret_cast<const uint4*>(row + 2ull * x0);
-      const uint4 a = CG ? __ldcg(q) : q[0];
-      const uint32_t w[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-      for (int i = 0; i < 4; i++) { v[2 * i] = w[i] & 0xffffu; v[2 * i + 1] = w[i] >> 16; }
-    } else {
-      const uint2* q = reinterpret_cast<const uint2*>(row + x0);
-      const uint2 a = CG ? __ldcg(q) : q[0];
-#pragma unroll
-      for (int i = 0; i < 4; i++) { v[i] = (a.x >> (8 * i)) & 0xffu; v[4 + i] = (a.y >> (8 * i)) & 0xffu; }
-    }
-    return;
-  }
-#pragma unroll
-  for (int i = 0; i < 8; i++)
-    v[i] = (uint32_t)i < nvalid ? (CG ? load_sample_cg(row, S, x0 + i) : load_sample(row, S, x0 + i)) : 0u;
-}
-
-template <uint32_t S>
-__device__ __forceinline__ void store8s(uint8_t* row, uint32_t x0, uint32_t nvalid, bool vec, const uint32_t (&v)[8]) {
-  if (vec && nvalid == 8) {
-    if constexpr (S == 4) {
-      uint4* q = reinterpret_cast<uint4*>(row + 4ull * x0);
-      q[0] = make_uint4(v[0], v[1], v[2], v[3]);
-      q[1] = make_uint4(v[4], v[5], v[6], v[7]);
-    } else if constexpr (S == 2) {
-      uint4* q = reinterpret_cast<uint4*>(row + 2ull * x0);
-      q[0] = make_uint4((v[0] & 0xffffu) | (v[1] << 16), (v[2] & 0xffffu) | (v[3] << 16),
-                        (v[4] & 0xffffu) | (v[5] << 16), (v[6] & 0xffffu) | (v[7] << 16));
-    } else {
-      uint2* q = reinterpret_cast<uint2*>(row + x0);
-      q[0] = make_uint2((v[0] & 0xffu) | ((v[1] & 0xffu) << 8) | ((v[2] & 0xffu) << 16) | (v[3] << 24),
-                        (v[4] & 0xffu) | ((v[5] & 0xffu) << 8) | ((v[6] & 0xffu) << 16) | (v[7] << 24));
-    }
-    return;
-  }
-#pragma unroll
-  for (int i = 0; i < 8; i++)
-    if ((uint32_t)i < nvalid) store_sample(row, S, x0 + i, v[i]);
-}
-
 __device__ __forceinline__ uint32_t warp_excl_scan(uint32_t v, uint32_t& total) {
   const uint32_t incl = warp_incl_scan(v);
   total = __shfl_sync(0xffffffffu, incl, 31);

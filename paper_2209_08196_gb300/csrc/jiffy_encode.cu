@@ -31,7 +31,8 @@
 //     row's slot; rows never wait for one another's sizes (sections differ a
 //     lot in cost, and an in-order prefix over rows would queue fast rows
 //     behind slow ones).
-//   k_sec_sizes one CTA per section: its bytes and nonzero count.
+//   k_sec_sizes one CTA per section: its bytes and nonzero count (calls of
+//               more than 1024 rows; else k_place adds them up).
 //   k_place     one CTA per section: offset (sum over the earlier sections),
 //               row table, frame and stream headers, and the copy of every
 //               row chunk from its slot to its place in the stream.
@@ -95,21 +96,6 @@ __device__ __forceinline__ uint32_t section_mode(const EncParams& p, const EncSe
   if (sg.frame0 + t == 0 || sg.force_mode == 0) return 0u;
   if (sg.force_mode == 1) return 1u;
   return p.cost[2 * sec + 1] < p.cost[2 * sec] ? 1u : 0u;
-}
-
-// Loads / stores 8 samples with the width fixed at compile time (S = 1, 2,
-// 4) or read at run time (S = 0).
-template <uint32_t S>
-__device__ __forceinline__ void ld8(const uint8_t* row, uint32_t s, uint32_t x0, uint32_t nv, bool vec,
-                                    uint32_t (&v)[8]) {
-  if constexpr (S == 0) load8<false>(row, s, x0, nv, vec, v);
-  else load8s<S, false>(row, x0, nv, vec, v);
-}
-template <uint32_t S>
-__device__ __forceinline__ void st8(uint8_t* row, uint32_t s, uint32_t x0, uint32_t nv, bool vec,
-                                    const uint32_t (&v)[8]) {
-  if constexpr (S == 0) store8(row, s, x0, nv, vec, v);
-  else store8s<S>(row, x0, nv, vec, v);
 }
 
 // ZigZag of a delta known to satisfy |d| < 2^30: with t = 2d, Eq. 1 gives
