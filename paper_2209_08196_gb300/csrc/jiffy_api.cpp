@@ -1064,14 +1064,16 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   }
   key.push_back(async ? 1u : 0u);
 
-  // Small calls run the rows kernel alone: the kernels around it cost about
+  // Small calls run the rows kernel alone: the kernels around it cost up to
   // 10 us a call (17 -> 28 us for 2 scans of 11 x 896, five attributes) and
-  // save a tenth of the rows' time, which is 10 us at some 16 million samples
-  // (100 scans of 128 x 2048, 131 million: 330 -> 290 us). They also take P
-  // runs apart, which pays for itself many times over in calls of many frames
-  // whose rows wait for one another (100 predicted scans of 64 x 489, 6
-  // million samples: 1.95 -> 0.12 ms), so long calls of a few thousand rows
-  // take them too.
+  // save up to a tenth of the rows' time (100 scans of 128 x 2048, 131 million
+  // samples: 330 -> 290 us when they came in). Without P frames the two forms
+  // meet between 39 million samples (82 us alone, 84 with them) and 65 million
+  // (129, 127). The line lies lower, at 16 million, for the P frames, which the
+  // host does not know of: the kernels take P runs apart, where rows that wait
+  // for one another cost about 19 us a frame (100 predicted scans of 64 x 489,
+  // 6 million samples: 1.95 -> 0.12 ms). For the same reason long calls of a
+  // few thousand rows take them too.
   const bool local = max_T == 1 || !(pixels >= (16ull << 20) || (max_T >= 32 && items >= 8192));
 
   jiffy::DecParams p{};
