@@ -74,12 +74,13 @@ __device__ __forceinline__ void store_sample(uint8_t* row, uint32_t s, uint32_t 
 }
 
 // Inclusive prefix sum over the warp; the shuffle itself says which lanes
-// have a source (no lane compares).
+// have a source (no lane compares). volatile: the whole warp takes part, so
+// the compiler may not move a step to where only some lanes use its result.
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1)
-    asm("{\n\t.reg .pred p;\n\t.reg .u32 t;\n\tshfl.sync.up.b32 t|p, %0, %1, 0, 0xffffffff;\n\t@p add.u32 %0, %0, t;\n\t}"
-        : "+r"(v) : "r"(o));
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .u32 t;\n\tshfl.sync.up.b32 t|p, %0, %1, 0, 0xffffffff;\n\t@p add.u32 %0, %0, t;\n\t}"
+                 : "+r"(v) : "r"(o));
   return v;
 }
 
