@@ -995,7 +995,9 @@ int decode_rows_launch(const DecParams& p, RowsLaunch* out) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) {
     void (*f)(DecParams) = rows_kernel(p, wpc);
-    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the limit is the kernel's, shared by all threads: always the same one,
+    // or a call of narrower rows takes it from another thread's launch)
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmemMax);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, (int)wpc * 32, smem);
   }
   if (e != cudaSuccess) return (int)e;

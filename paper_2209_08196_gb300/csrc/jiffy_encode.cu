@@ -1076,7 +1076,9 @@ constexpr size_t kRowsSmemMax = 227 * 1024;
 template <int WPC>
 static cudaError_t rows_occupancy(size_t smem, bool staged, int* per_sm) {
   auto f = staged ? k_encode<WPC, true> : k_encode<WPC, false>;
-  cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (the limit is the kernel's, shared by all threads and launches: always the
+  // same one, or a call of narrower rows takes it from another's launch)
+  cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmemMax);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, f, WPC * 32, smem);
 }
@@ -1117,7 +1119,8 @@ int launch_encode(const EncParams& p, void* stream, void* const* ev) {
   int rc = encode_rows_launch(p, &rl);
   if (rc != 0) return rc;
   const size_t s_place = 4ull * kMaxH + 4ull * zmask_blocks(kMaxH, kMaxW);  // row starts, block starts
-  cudaError_t e = cudaFuncSetAttribute(k_trial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_trial);
+  cudaError_t e = cudaFuncSetAttribute(k_trial, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)trial_smem_bytes_host(kMaxW));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_place, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_place);
   if (e != cudaSuccess) return (int)e;
   auto mark = [&](int i) {
@@ -1128,14 +1131,10 @@ int launch_encode(const EncParams& p, void* stream, void* const* ev) {
   mark(1);
   // rows of narrow segments first, with shared memory (and so occupancy) for
   // their own width, then the wider ones: one rows launch per width class
-  // (each launch sets its own shared-memory limit first: resolving another
-  // launch's configuration changes it)
   auto rows = [&](const EncParams& q, const RowsLaunch& r) -> cudaError_t {
     const size_t smem = (size_t)r.wpc * enc_warp_layout(q.max_W).bytes;
     void (*f)(EncParams) = q.staged ? (r.wpc == 4 ? k_encode<4, true> : r.wpc == 2 ? k_encode<2, true> : k_encode<1, true>)
                                     : (r.wpc == 4 ? k_encode<4, false> : r.wpc == 2 ? k_encode<2, false> : k_encode<1, false>);
-    cudaError_t ce = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (ce != cudaSuccess) return ce;
     f<<<r.grid, r.wpc * 32, smem, st>>>(q);
     return cudaGetLastError();
   };
