@@ -391,7 +391,12 @@ jiffy_status check_distinct(const std::vector<jiffy_stream*>& ss) {
 // JIFFY_TUNE_CACHE: one line per shape class, "jiffy-tune 1 <device> <n>
 // <n key words> <warps per CTA> <CTAs per SM> <items per ticket>", device =
 // SM count * 1000 + compute capability (lines of another device are ignored;
-// a configuration that does not fit falls back to the automatic one).
+// a configuration that does not fit falls back to the automatic one). The key
+// says what was timed: role, widest row, log2 of the rows, whether the staged
+// instance runs, the decoder's form, and kTunedKernels, which is raised when
+// the rows kernels change, so that what was timed on others is not taken.
+constexpr uint32_t kTunedKernels = 2;
+
 using TuneKey = std::pair<uint32_t, std::vector<uint32_t>>;
 
 const char* tune_cache_path() {
@@ -697,7 +702,7 @@ jiffy_status enqueue_encode(Workspace& ws, std::vector<EncJob>& jobs, cudaStream
   uint32_t* ib = reinterpret_cast<uint32_t*>(h + u_ib);
   uint32_t* sb = reinterpret_cast<uint32_t*>(h + u_sb);
   std::vector<uint64_t> key{1, n, (uint64_t)(uintptr_t)d, (uint64_t)(uintptr_t)h};
-  std::vector<uint32_t> sig{1, max_W, log2_ceil(items)};
+  std::vector<uint32_t> sig{1, max_W, log2_ceil(items), kTunedKernels};
   uint32_t staged = 0, withhold = 0;
   uint32_t item_base = 0, sec_base = 0;
   // segment order: streams of rows up to kNarrowW columns first, so that the
@@ -944,6 +949,18 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   if (check_distinct(ss) != JIFFY_OK) return JIFFY_ERR_INVALID_ARG;
   if (items > 0x7fffffffull) return JIFFY_ERR_INVALID_ARG;
 
+  // Small calls run the rows kernel alone: the kernels around it cost up to
+  // 10 us a call (17 -> 28 us for 2 scans of 11 x 896, five attributes) and
+  // save up to a tenth of the rows' time (100 scans of 128 x 2048, 131 million
+  // samples: 330 -> 290 us when they came in). Without P frames the two forms
+  // meet between 39 million samples (82 us alone, 84 with them) and 65 million
+  // (129, 127). The line lies lower, at 16 million, for the P frames, which the
+  // host does not know of: the kernels take P runs apart, where rows that wait
+  // for one another cost about 19 us a frame (100 predicted scans of 64 x 489,
+  // 6 million samples: 1.95 -> 0.12 ms). For the same reason long calls of a
+  // few thousand rows take them too.
+  const bool local = max_T == 1 || !(pixels >= (16ull << 20) || (max_T >= 32 && items >= 8192));
+
   Carver up;
   const size_t u_seg = up.take(sizeof(jiffy::DecSeg) * n), u_ib = up.take(4ull * n), u_sb = up.take(4ull * n),
                u_cb = up.take(4ull * n);
@@ -995,7 +1012,7 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   uint32_t* sbk = reinterpret_cast<uint32_t*>(h + u_sb);
   uint32_t* cbk = reinterpret_cast<uint32_t*>(h + u_cb);
   std::vector<uint64_t> key{2, n, (uint64_t)(uintptr_t)d, (uint64_t)(uintptr_t)h};
-  std::vector<uint32_t> sig{2, max_W, log2_ceil(items)};
+  std::vector<uint32_t> sig{2, max_W, log2_ceil(items), local ? 1u : 0u, kTunedKernels};
   uint32_t staged = 0, withhold = 0;
   uint32_t item_base = 0, sec_base = 0, chain_base = 0;
   for (uint32_t i = 0; i < n; i++) {
@@ -1063,18 +1080,6 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
     if (j.async) key.push_back((uint64_t)(uintptr_t)j.frame_offsets);
   }
   key.push_back(async ? 1u : 0u);
-
-  // Small calls run the rows kernel alone: the kernels around it cost up to
-  // 10 us a call (17 -> 28 us for 2 scans of 11 x 896, five attributes) and
-  // save up to a tenth of the rows' time (100 scans of 128 x 2048, 131 million
-  // samples: 330 -> 290 us when they came in). Without P frames the two forms
-  // meet between 39 million samples (82 us alone, 84 with them) and 65 million
-  // (129, 127). The line lies lower, at 16 million, for the P frames, which the
-  // host does not know of: the kernels take P runs apart, where rows that wait
-  // for one another cost about 19 us a frame (100 predicted scans of 64 x 489,
-  // 6 million samples: 1.95 -> 0.12 ms). For the same reason long calls of a
-  // few thousand rows take them too.
-  const bool local = max_T == 1 || !(pixels >= (16ull << 20) || (max_T >= 32 && items >= 8192));
 
   jiffy::DecParams p{};
   p.local = local ? 1u : 0u;

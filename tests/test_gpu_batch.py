@@ -428,3 +428,47 @@ def test_many_stream_workload_sampled_against_oracle():
         for t in range(c.n_scans):
             for a, (s, _) in enumerate(at):
                 assert np.array_equal(to_np(dec_planes[i][a][t], s), ref_planes[t][a]), (i, t, a)
+
+
+def test_tuned_launches_are_kept_apart_by_the_decoders_form():
+    # 31 and 32 frames of 256 rows fall into the same class of widest row and
+    # row count, but the longer call runs the kernels around the rows
+    # (8192 rows and 32 frames): it is tuned by itself
+    rng = np.random.default_rng(29)
+    H, W, attrs = 256, 40, [(2, 1)]
+    b, plain = J.jiffy_batch_create(), J.jiffy_batch_create()
+    J.jiffy_batch_set_autotune(b, True)
+    for call, T in enumerate((31, 32)):
+        planes = to_dev(np.stack([s[0] for s in make_scans(rng, H, W, attrs, T)]))
+        out = torch.zeros(J.jiffy_max_encoded_size(H, W, attrs, T), dtype=torch.uint8, device="cuda")
+        enc = J.jiffy_stream_create(J.JIFFY_ENCODER, H, W, attrs)
+        dec = J.jiffy_stream_create(J.JIFFY_DECODER, H, W, attrs)
+        (n, offs), = J.jiffy_encode_batch(plain, [enc], [[planes]], [out])
+        got = torch.zeros_like(planes)
+        J.jiffy_decode_batch(b, [dec], [out], [n], [offs], [[got]])
+        assert torch.equal(got, planes), T
+        assert J.jiffy_batch_info(b)["tunings"] == call + 1, T
+
+
+def test_tune_cache_entries_of_other_kernels_are_not_taken(tmp_path, monkeypatch):
+    # entries whose key does not name the present rows kernels: role, widest
+    # row, log2 of the rows, staged
+    path = tmp_path / "tune.txt"
+    p = torch.cuda.get_device_properties(0)
+    dev = p.multi_processor_count * 1000 + p.major * 10 + p.minor
+    path.write_text("".join("jiffy-tune 1 %d 4 %d 1024 5 0 1 1 1\n" % (dev, role) for role in (1, 2)))
+    monkeypatch.setenv("JIFFY_TUNE_CACHE", str(path))
+    rng = np.random.default_rng(30)
+    H, W, attrs, T = 16, 1024, [(4, 1)], 2
+    planes = to_dev(np.stack([s[0] for s in make_scans(rng, H, W, attrs, T)]))
+    out = torch.zeros(J.jiffy_max_encoded_size(H, W, attrs, T), dtype=torch.uint8, device="cuda")
+    enc = J.jiffy_stream_create(J.JIFFY_ENCODER, H, W, attrs)
+    dec = J.jiffy_stream_create(J.JIFFY_DECODER, H, W, attrs)
+    b = J.jiffy_batch_create()
+    J.jiffy_batch_set_autotune(b, True)
+    (n, offs), = J.jiffy_encode_batch(b, [enc], [[planes]], [out])
+    assert J.jiffy_batch_info(b)["tunings"] == 1
+    got = torch.zeros_like(planes)
+    J.jiffy_decode_batch(b, [dec], [out], [n], [offs], [[got]])
+    assert J.jiffy_batch_info(b)["tunings"] == 2
+    assert torch.equal(got, planes)
