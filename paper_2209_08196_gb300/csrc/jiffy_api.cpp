@@ -1045,7 +1045,7 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
     g.frame0 = s->frame;
     g.fhdr = frame_header_bytes(A);
     g.check_shdr = s->frame == 0;
-    g.clear_err = j.async ? 0u : 1u;  // (where nothing else clears it)
+    g.clear_err = j.async ? 0u : 1u;  // (an enqueue-only call's adds up until the wait)
     g.item_base = item_base;
     g.chain_base = chain_base;
     g.attrs = s->d_attrs;
@@ -1117,12 +1117,13 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   if (!up_same && async && record_ev(ws.uploaded, st) != cudaSuccess) return JIFFY_ERR_CUDA;
 
   auto enqueue = [&](cudaStream_t s, const jiffy::DecParams& pp, void* const* evs) -> int {
-    // Long calls clear these words in their first kernel. Synchronous ones
-    // clear them here too: with the table's copy straight ahead of that kernel
-    // the call was seen to wait for bulk copies of other streams, and a
-    // pipeline with 419 MB each way in flight beside its calls took 2.97 ms
-    // instead of 2.72 a step; the clear costs 3 us a call.
-    if (local || !async) {
+    // Long calls clear these words in their first kernel. Small ones clear them
+    // here, and so do long blocking ones whose kernels are timed: a timing event
+    // straight behind the table's copy takes its time, it seems, on the copy
+    // engine, where it waits for other streams' bulk copies (a pipeline with 419
+    // MB each way in flight beside its calls: 2.90 ms a step, 2.64 with the
+    // clear in between, and 2.64 either way without timing).
+    if (local || (evs && !async)) {
       const cudaError_t ce = cudaMemsetAsync(d + o_zero, 0, zero_bytes, s);
       if (ce != cudaSuccess) return (int)ce;
     }
