@@ -116,3 +116,175 @@ def test_batch_of_single_and_several_frames(sensors):
         for t in range(T):
             for k, (s, _) in enumerate(attrs):
                 assert np.array_equal(to_np(got[k][t], s), want[t][k]), (H, W, t, k)
+
+
+# Calls large enough for the kernels around the rows, whose state nothing but
+# those kernels clears when they are enqueue-only, and malformed ones among
+# them. Runs of two P frames are added by rows that wait, long ones behind the
+# rows (3000 rows per frame of the longest run).
+BIG = (128, 65, [(2, 1), (1, 1)])
+ZERO_ROW = 7  # a row without samples: its chunk is one class word
+
+
+def predicted(rng, T, run):
+    """Frames of noise, each followed by `run` near copies of it (coded P)."""
+    H, W, attrs = BIG
+    out = []
+    for t in range(T):
+        if t % (run + 1) == 0:
+            base = [rng.integers(1, 1 << (8 * s), size=(H, W)) for s, _ in attrs]
+        planes = []
+        for (s, _), b in zip(attrs, base):
+            x = np.clip(b + rng.integers(-1, 2, size=b.shape), 1, (1 << (8 * s)) - 1)
+            x[rng.random(x.shape) < 0.1] = 0
+            x[ZERO_ROW] = 0
+            planes.append(x.astype(DT[s]))
+        out.append(planes)
+    return out
+
+
+def coded(ref, refd, scans, waits):
+    """(stream bytes, frame offsets, planes) of a call's scans by the oracle;
+    waits: whether the rows of its P runs wait for one another."""
+    H, W, attrs = BIG
+    parts = [ref.encode(s, return_modes=True) for s in scans]
+    longest = 0
+    for a in range(len(attrs)):
+        run = 0
+        for t, (_, modes) in enumerate(parts):
+            run = run + 1 if t and modes[a] == 1 else 0
+            longest = max(longest, run)
+    rows = len(scans) * len(attrs) * H
+    assert len(scans) >= 32 and rows >= 8192 and longest >= 2
+    assert (longest * 3000 <= rows) == waits, longest
+    ends = np.cumsum([len(b) for b, _ in parts]).tolist()
+    return b"".join(b for b, _ in parts), ends, [refd.decode(b)[0] for b, _ in parts]
+
+
+def on_gpu(data):
+    return torch.from_numpy(np.frombuffer(bytes(data), dtype=np.uint8).copy()).cuda()
+
+
+def check_planes(planes, want, what=""):
+    for t, w in enumerate(want):
+        for k, (s, _) in enumerate(BIG[2]):
+            assert np.array_equal(to_np(planes[k][t], s), w[k]), (what, t, k)
+
+
+def test_enqueued_calls_clear_what_the_calls_before_them_left():
+    # four enqueue-only calls in flight on one handle before the wait, the
+    # P runs of some summed and of some waited for, then all of them again
+    H, W, attrs = BIG
+    rng = np.random.default_rng(41)
+    ref, refd = oracle.Codec(H, W, attrs), oracle.Codec(H, W, attrs)
+    dec = J.jiffy_stream_create(J.JIFFY_DECODER, H, W, attrs)
+    calls = []
+    for i, (T, run) in enumerate(((40, 1000), (33, 2), (40, 2), (64, 1000))):
+        data, ends, want = coded(ref, refd, predicted(rng, T, run), run == 2)
+        offs = torch.tensor([16 + 8 * len(attrs) if i == 0 else 0] + ends, dtype=torch.int64, device="cuda")
+        calls.append((on_gpu(data), offs, want))
+    for _ in range(2):
+        J.jiffy_stream_reset(dec)
+        outs = []
+        for src, offs, want in calls:
+            outs.append([torch.zeros((len(want), H, W), dtype=TORCH_DT[s], device="cuda") for s, _ in attrs])
+            J.jiffy_decode_seq_async(dec, src, offs, outs[-1])
+        J.jiffy_stream_wait(dec)
+        for i, ((_, _, want), planes) in enumerate(zip(calls, outs)):
+            check_planes(planes, want, i)
+
+
+def damaged(data, ends, kind, t):
+    """The stream with frame t of its call damaged (attribute 0)."""
+    H, W, attrs = BIG
+    b = bytearray(data)
+    f = ends[t - 1]                          # frame t's header
+    sec = f + 8 + 12 * len(attrs)            # its first section: the row table
+    end = lambda r: int.from_bytes(b[sec + 8 * r:sec + 8 * r + 4], "little")  # noqa: E731
+    chunk = lambda r: sec + 8 * H + (end(r - 1) if r else 0)  # noqa: E731
+    if kind == "mode":
+        b[f + 8] = 2
+    elif kind == "section bytes":
+        b[f + 12] ^= 4
+    elif kind == "row end":
+        b[sec + 8 * 5] ^= 8
+    elif kind == "row end far away":
+        b[sec + 8 * 5:sec + 8 * 5 + 4] = (0xFFFFFFF0).to_bytes(4, "little")
+    elif kind == "invalid class":
+        b[chunk(5)] = 0xFF
+    elif kind == "literals for every word":
+        b[chunk(5)] = 0x2A
+    elif kind == "literals past the chunk":
+        assert end(ZERO_ROW) - end(ZERO_ROW - 1) == 4
+        b[chunk(ZERO_ROW)] = 0x2A
+    else:  # a block of 40 bits
+        cls = b[chunk(5)]
+        lits = sum((cls >> (2 * j)) & 3 == 2 for j in range(3))
+        b[chunk(5) + 4 * (1 + lits)] = 40
+    return b
+
+
+KINDS = ["mode", "section bytes", "row end", "row end far away", "invalid class", "literals for every word",
+         "literals past the chunk", "block width"]
+
+
+@pytest.mark.parametrize("run", [2, 1000])
+@pytest.mark.parametrize("kind", KINDS)
+def test_damaged_frames_inside_a_run_are_refused(kind, run):
+    # in a P frame, and in an I or P frame whose successor is coded P; the
+    # decoder goes on with the undamaged stream, blocking and enqueue-only
+    H, W, attrs = BIG
+    T = 40
+    rng = np.random.default_rng(run)
+    data, ends, want = coded(oracle.Codec(H, W, attrs), oracle.Codec(H, W, attrs), predicted(rng, T, run), run == 2)
+    offs = [16 + 8 * len(attrs)] + ends
+    d_offs = torch.tensor(offs, dtype=torch.int64, device="cuda")
+    dec = J.jiffy_stream_create(J.JIFFY_DECODER, H, W, attrs)
+    good = on_gpu(data)
+    for t in (6, 7):
+        b = damaged(data, ends, kind, t)
+        refd = oracle.Codec(H, W, attrs)
+        with pytest.raises(oracle.OracleError):
+            for k in range(t + 1):
+                refd.decode(bytes(b[(ends[k - 1] if k else 0):ends[k]]))
+        bad = on_gpu(b)
+        planes = [torch.zeros((T, H, W), dtype=TORCH_DT[s], device="cuda") for s, _ in attrs]
+        J.jiffy_stream_reset(dec)
+        with pytest.raises(J.JiffyError) as ei:
+            J.jiffy_decode_seq(dec, bad, bad.numel(), offs, planes)
+        assert ei.value.name == "JIFFY_ERR_CORRUPT"
+        assert J.jiffy_stream_frame_index(dec) == 0
+        J.jiffy_decode_seq(dec, good, good.numel(), offs, planes)
+        check_planes(planes, want, "blocking")
+        planes = [torch.zeros_like(p) for p in planes]
+        J.jiffy_stream_reset(dec)
+        J.jiffy_decode_seq_async(dec, bad, d_offs, planes)
+        with pytest.raises(J.JiffyError) as ei:
+            J.jiffy_stream_wait(dec)
+        assert ei.value.name == "JIFFY_ERR_CORRUPT"
+        J.jiffy_stream_reset(dec)
+        J.jiffy_decode_seq_async(dec, good, d_offs, planes)
+        J.jiffy_stream_wait(dec)
+        check_planes(planes, want, "enqueue-only")
+
+
+@pytest.mark.parametrize("run", [2, 1000])
+def test_bounded_wait_of_a_large_call_runs_out_and_the_stream_recovers(run):
+    # one row withholds its completion flag (host-side hook; the rows of every
+    # P run then wait): the same row of the next frame gives up after the
+    # bounded wait, the rest of the call goes on, the stream's state is as
+    # before and the same frames decode next
+    H, W, attrs = BIG
+    T = 40
+    rng = np.random.default_rng(100 + run)
+    data, ends, want = coded(oracle.Codec(H, W, attrs), oracle.Codec(H, W, attrs), predicted(rng, T, run), run == 2)
+    src, offs = on_gpu(data), [16 + 8 * len(attrs)] + ends
+    planes = [torch.zeros((T, H, W), dtype=TORCH_DT[s], device="cuda") for s, _ in attrs]
+    dec = J.jiffy_stream_create(J.JIFFY_DECODER, H, W, attrs)
+    J.jiffy_stream_test_withhold_row(dec, 3 * H + 5)  # attribute 0, scan 3 (scan 4 is coded P), row 5
+    with pytest.raises(J.JiffyError) as ei:
+        J.jiffy_decode_seq(dec, src, len(data), offs, planes)
+    assert ei.value.name == "JIFFY_ERR_TIMEOUT"
+    assert J.jiffy_stream_frame_index(dec) == 0
+    J.jiffy_decode_seq(dec, src, len(data), offs, planes)
+    check_planes(planes, want)
