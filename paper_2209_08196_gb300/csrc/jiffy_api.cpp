@@ -949,16 +949,20 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   if (check_distinct(ss) != JIFFY_OK) return JIFFY_ERR_INVALID_ARG;
   if (items > 0x7fffffffull) return JIFFY_ERR_INVALID_ARG;
 
-  // Small calls run the rows kernel alone: the kernels around it cost up to
-  // 10 us a call (17 -> 28 us for 2 scans of 11 x 896, five attributes) and
-  // save up to a tenth of the rows' time (100 scans of 128 x 2048, 131 million
-  // samples: 330 -> 290 us when they came in). Without P frames the two forms
-  // meet between 39 million samples (82 us alone, 84 with them) and 65 million
-  // (129, 127). The line lies lower, at 16 million, for the P frames, which the
-  // host does not know of: the kernels take P runs apart, where rows that wait
-  // for one another cost about 19 us a frame (100 predicted scans of 64 x 489,
-  // 6 million samples: 1.95 -> 0.12 ms). For the same reason long calls of a
-  // few thousand rows take them too.
+  // Small calls run the rows kernel alone. Blocking calls in us, one kernel /
+  // with the kernels around it:
+  //   predicted, 64 x 489 range: 4 frames 53 / 48, 8 74 / 51, 16 123 / 59,
+  //     32 222 / 63, 100 628 / 96 (6 us a frame of the run in the one form)
+  //   none predicted: 128 x 2048 range, 8 frames 45 / 57, 64 79 / 78, 250
+  //     203 / 199; 41 x 2931 range, 178 frames 150 / 155; 128 x 2048 five
+  //     attributes, 13 frames 76 / 74, 40 146 / 142
+  // So without P frames the kernels cost up to 12 us and the forms meet at some
+  // 16 million samples, where the line lies (5 us lost at worst above it); with
+  // P frames they save 6 us a frame, and the host does not know which it has.
+  // Calls of 32 frames and more of 8192 rows and more, which lose little
+  // without P frames, take them too (64 x 489, two attributes, 64 frames:
+  // 414 / 81 predicted, 57 / 60 not). Predicted calls below both lines take
+  // the 6 us a frame.
   const bool local = max_T == 1 || !(pixels >= (16ull << 20) || (max_T >= 32 && items >= 8192));
 
   Carver up;
@@ -1090,7 +1094,6 @@ jiffy_status enqueue_decode(Workspace& ws, std::vector<DecJob>& jobs, cudaStream
   p.seg_item_base = reinterpret_cast<const uint32_t*>(d + o_up + u_ib);
   p.secs = reinterpret_cast<jiffy::DecSec*>(d + o_secs);
   p.n_chains = chains;
-  p.max_T = max_T;
   p.seg_chain_base = reinterpret_cast<const uint32_t*>(d + o_up + u_cb);
   p.chain_p = reinterpret_cast<uint32_t*>(d + o_chp);
   p.done = reinterpret_cast<uint32_t*>(d + o_done);

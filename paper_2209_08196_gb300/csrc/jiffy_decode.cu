@@ -150,8 +150,10 @@ __device__ __forceinline__ DecSec find_section(const DecSeg& sg, uint32_t t, uin
 // segment (a chain), a thread per section of it. It finds and checks the
 // sections, so that the rows, which are many per section, only read the
 // result; left to the rows it takes each of them three dependent rounds of
-// loads (replaying 100 scans of 128 x 2048: 329 us of rows, 278 us without). It also decides how the chain's P frames are added
-// up, and clears what the call counts with (no clearing pass of its own).
+// loads (replaying 100 scans of 128 x 2048: 329 us of rows, 278 us without,
+// both before the unpacking was rewritten). It also decides how the chain's P
+// frames are added up, and clears what the call counts with: the ticket, the
+// done flags that are waited for, a blocking call's error words.
 //
 // P frames (Sec. III-D) after a call's first frame need the same row of the
 // frame before. Either their rows wait for it (kLinkWait), which is free as
@@ -283,8 +285,9 @@ __device__ __forceinline__ uint32_t frame_mode(const DecParams& p, const DecSeg&
 
 // k_dec_masks, ahead of the rows of a call with segments of several frames:
 // the masks of P frames are chained by XOR (Sec. III-D). Left to the rows,
-// every frame of a P run waited for the whole decode of the frame before it
-// (19 us a frame at 64 x 489). Here CTAs take the rows of an attribute:
+// every frame of a P run waits for the frame before it (6 us a frame at 64 x
+// 489 with masks and pixels waited for apart, 19 us when it waited for the
+// whole decode). Here CTAs take the rows of an attribute:
 // a thread reads the coded mask words of one frame, and the frames are
 // combined by a scan over the lanes that restarts at every I frame (and over
 // the CTA's 8 warps through shared memory, 256 frames at a time). The masks

@@ -4,8 +4,8 @@
 // segments of the call), all in parallel: the P prediction of scan t uses the
 // *input* of scan t-1 (Sec. III-D), so no scan waits for another's output.
 // Launches:
-//   k_trial     one warp per (section, test row): I and P residuals of the
-//               scanline, delta chained across the test rows, priced with
+//   k_trial     one warp per (section, test row, mode): the scanline's I or P
+//               residuals, delta chained across the test rows, priced with
 //               the block-width choice below; the bytes add up per section
 //               and mode (trial compression, mask excluded, Sec. III-E, IV-E).
 //   k_encode    one warp per row item (scan, attribute, row), items taken in
@@ -32,8 +32,9 @@
 //     lot in cost, and an in-order prefix over rows would queue fast rows
 //     behind slow ones).
 //   k_sec_sizes one CTA per section: its bytes and nonzero count (calls of
-//               more than 1024 rows; else k_place adds them up).
-//   k_place     one CTA per section: offset (sum over the earlier sections),
+//               more than 1024 rows or with Zstandard masks; else k_place adds
+//               them up).
+//   k_place     four CTAs per section: offset (sum over the earlier sections),
 //               row table, frame and stream headers, and the copy of every
 //               row chunk from its slot to its place in the stream.
 #include "jiffy_device.cuh"
@@ -589,8 +590,8 @@ __device__ __forceinline__ uint32_t code_step(uint32_t* zb, uint32_t s0, uint32_
 
 // ----------------------------------------------------------------------------
 // k_trial: Sec. III-E. For sections with a predecessor and no forced mode,
-// one warp per test row floor((2k+1)H/(2L)) (de-duplicated): the I and P
-// residuals of the row, delta-chained from the last residual of the earlier
+// a warp for I and one for P per test row floor((2k+1)H/(2L)) (de-duplicated):
+// the residuals of the row, delta-chained from the last residual of the earlier
 // test rows (the test rows' residuals form one flat vector starting from 0),
 // priced per block. cost[2 sec + mode] += the row's block bytes.
 // ----------------------------------------------------------------------------
@@ -849,7 +850,7 @@ __global__ void __launch_bounds__(WPC * 32, 24 / WPC) k_encode(EncParams p) {
 // k_sec_sizes: one CTA per section (scan t, attribute a): its bytes (row
 // table + row chunks) and nonzero count (larger calls; adding them up in
 // k_encode, two atomics a row, made that 20 us longer where this takes 4).
-// k_place: one CTA per section: the section's offset in the stream (sum over
+// k_place: four CTAs per section: the section's offset in the stream (sum over
 // the segment's earlier sections), its row table (end offsets + carries),
 // the copy of each row chunk from its slot and, for attribute 0, the frame
 // header and frame offset; section 0 also writes the stream header. Every

@@ -89,7 +89,7 @@ struct DecSeg {
   uint32_t frame0;
   uint32_t fhdr;
   uint32_t check_shdr;           // validate the stream header at in[0]
-  uint32_t clear_err;            // the error word belongs to this call: cleared first
+  uint32_t clear_err;            // 1: a blocking call, the error word is its own and cleared first
   uint32_t item_base;            // first global row item of the segment
   uint32_t chain_base;           // first chain of the segment (it has A)
   const AttrDev* attrs;
@@ -132,13 +132,12 @@ struct DecParams {
   uint32_t n_chains;             // chains of all segments
   const uint32_t* seg_chain_base;// [n_seg] (search key for chains)
   uint32_t* chain_p;             // [n_chains] kLink* of the chain, by the call's first kernel
-  uint32_t max_T;                // most frames of a segment
   uint32_t* done;                // [n_items] row-done flags (of the chains that wait)
   uint32_t* masks;               // decoded zero masks, nw words per row item (frames coded P and those before them)
   uint32_t* ticket;
   uint32_t wpc;                  // warps per CTA (1, 2, 4, 8; 0 = by shared memory)
   uint32_t ctas_per_sm;          // resident CTAs per SM (0 = occupancy limit)
-  uint32_t items_per_ticket;     // row items a warp takes per ticket (0 = 4)
+  uint32_t items_per_ticket;     // row items a warp takes per ticket (0 = 1)
   uint32_t staged;               // as in EncParams
   uint32_t withhold;             // test hook: 1 + the row item that does not publish its done flag (0: none)
   // Zstandard mask sections (null when no segment codes its mask that way)

@@ -163,7 +163,6 @@ extern "C" jiffy_status jiffy_decode_frame_noalloc(const void* in, size_t in_len
   p.seg_item_base = reinterpret_cast<const uint32_t*>(scratch + kOffSegKey);
   p.done = reinterpret_cast<uint32_t*>(scratch + kOffDone);
   p.ticket = reinterpret_cast<uint32_t*>(scratch + kOffTicket);
-  p.max_T = 1;
   p.local = 1;
   p.staged = stages ? 1u : 0u;  // the decoder instance that reads the stage switches
   if (launch_decode(p, cuda_stream, nullptr) != 0) return JIFFY_ERR_CUDA;

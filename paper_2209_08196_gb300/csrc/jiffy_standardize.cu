@@ -28,8 +28,9 @@
 // Two launches per call of up to 256 scans: k_std_points (one thread per
 // point, one grid row per scan: pixel and an atomicMin of the key (R << 32 |
 // index in the scan) into a per-pixel word, L2-resident for a few scans) and
-// k_std_pixels (one thread per pixel of every scan, grid-stride: the winning
-// point's range and attributes, and the key word reset for the next call).
+// k_std_pixels (a warp per 128 pixels of a scan, four a lane, grid-stride: the
+// winning point's range and attributes, and the key word reset for the next
+// call).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -178,10 +179,10 @@ __device__ __noinline__ uint32_t exact_pixel(const StdParams& p, long long X, lo
 }
 
 // The same pixel from float32 angles, where they decide it. A CORDIC angle is
-// within 1.5e-7 rad of the true one (30 truncated steps on 28-bit vectors and
-// more, 30 rounded table entries), a float32 one within 1.2e-6 rad (atan2f: 3
-// ulp, 7.2e-7 at half a turn; inputs and scaling 4e-7): together less than
-// 1000 units of 2^-32 turn. So where the pixel is the same over kMargin units
+// within 1.5e-7 rad of the true one by its error bound (30 truncated steps on
+// 28-bit vectors and more, 30 rounded table entries; below 6e-8 where tested),
+// a float32 one within 1.2e-6 rad (atan2f: 3 ulp, 7.2e-7 at half a turn;
+// inputs and scaling 4e-7): together less than 1000 units of 2^-32 turn. So where the pixel is the same over kMargin units
 // either side of the float angle, the CORDIC angle falls into it too. About 1
 // point in 300 of a 128 x 2048 image is closer to an edge than that (returns
 // false) and goes to exact_pixel. With two CORDICs for every point (935

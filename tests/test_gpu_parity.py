@@ -379,10 +379,10 @@ def test_bounded_wait_runs_out_and_the_stream_recovers():
 
 
 def test_encoder_carry_wait_runs_out_and_the_stream_recovers():
-    # only row 0 has nonzero samples, so a row r >= 5 finds no kept sample
-    # among the 2048 samples before it (the direct search) and its delta
-    # carry comes from the look-back over the earlier rows' last residuals;
-    # one row withholds its status (host-side hook), the rows after it give
+    # only row 0 has nonzero samples, so a row r >= 2 finds no kept sample
+    # among the last 256 of the row before it (the direct search) and its
+    # delta carry comes from the look-back over the earlier rows' last
+    # residuals; one row withholds its status (host-side hook), the rows after it give
     # up after the bounded wait, the call reports a timeout and leaves the
     # stream as it was
     rng = np.random.default_rng(78)
