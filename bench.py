@@ -492,7 +492,7 @@ def batched_leg(J, torch, dev, local, steps, warmup, n_streams=256, n_scans=8, b
             "auto_launch_gpoints_s": px / (ms_auto / 1e3) / 1e9,
             "auto_launch": {k: info_auto[k] for k in ("warps_per_cta", "ctas_per_sm", "items_per_ticket", "grid")},
             "graph_replays": info["graph_replays"], "tunings": info["tunings"], "gen_s": t_gen,
-            "launches_per_step": 5}
+            "launches_per_step": 9}  # encode 5 (narrow and wide rows apart), decode 4
 
 
 def serve_leg(J, torch, dev, local, seconds, sat_seconds, n_sensors=512, base_seed=5000):
@@ -736,7 +736,7 @@ def small_stream_leg(J, torch, dev, local, steps=200, warmup=5):
                           "k_decode": 1e3 * kd[0]},
             "graphs": "each call's launch sequence replayed from a CUDA graph (not with profiling on)",
             "l2": "cold: 256 MiB write before each step; hot: back-to-back steps, inputs in L2",
-            "launches_per_step": 5}
+            "launches_per_step": 4}  # encode 3 (1024 rows: no size kernel), decode 1
 
 
 def _zstd():
